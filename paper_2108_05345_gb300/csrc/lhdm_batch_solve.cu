@@ -15,6 +15,8 @@ __global__ void __launch_bounds__(NT, 1) lhdm_solve_batch_kernel(const BatchItem
   I.phase_ns = nullptr;
   I.trace = nullptr;
   I.trace_cap = 0;
+  const TcState tc = tc_open();
+  unsigned mpar = 0u;  // parities of tc's barriers, from instance to instance
   for (;;) {
     if (threadIdx.x == 0) s_k = atomicAdd(queue, 1);
     __syncthreads();
@@ -26,7 +28,16 @@ __global__ void __launch_bounds__(NT, 1) lhdm_solve_batch_kernel(const BatchItem
     bind_item(I, it);
     CtaTeam tm{0, 1};
     Engine<CtaTeam> e(tm, I, dyn);
+    e.mbs = tc.mbs;
+    e.tmem = tc.tmem;
+    e.mpar = mpar;
     e.run();
+    mpar = e.mpar;
+    if (e.tc_failed) {
+      tc_reset(tc);
+      mpar = 0u;
+    }
     __syncthreads();
   }
+  tc_close(tc);
 }

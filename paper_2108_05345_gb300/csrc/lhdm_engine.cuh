@@ -122,9 +122,9 @@ struct Inst {
   double* accb;   // ceil(cap/TB) x TB slab accumulations of the pipelined solve
   int* tflag;     // ceil(cap/TB) block flags, ceil(cap/TB) * TB/SLAB slab flags, ceil(cap/TB) * INV_PARTS inverse flags
   unsigned long long* amask;  // KM acceptance masks
-  unsigned* Vd;   // panel reflectors as 7-bit digits: m rows x ND planes x 16 words (bf16 pairs,
-                  // 16-byte chunk c of row r at c ^ (r & 7)), null: none
-  int* Ver;       // m: row scale exponents of Vd (|V(r, :)| < 2^Ver[r])
+  unsigned* Vd;   // panel reflectors as 7-bit digits (bf16): groups of 8 rows, per group ND digits
+                  // x kdig / 8 blocks of 8 rows x 8 reflectors; null: none
+  int* Ver;       // row scale exponents of Vd (|V(r, :)| < 2^Ver[r + (nP & 7)])
   double* phase_ns;           // 2 NPHASE + 1 (may be null): phase times, phase flops,
                               // bf16 MMAs of the tensor-core commit
   int* trace;                 // 6 ints per outer step (may be null)
@@ -274,13 +274,17 @@ __device__ __forceinline__ void sign2(bool nega, bool negb, unsigned& sg, unsign
   sg = (nega ? 0xBF80u : 0x3F80u) | ((negb ? 0xBF80u : 0x3F80u) << 16);
   nb = (nega ? 0x4300u : 0xC300u) | ((negb ? 0x4300u : 0xC300u) << 16);
 }
+// p s + n on bf16 pairs
+__device__ __forceinline__ unsigned bf16x2_fma(unsigned p, unsigned s, unsigned n) {
+  unsigned r;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(p), "r"(s), "r"(n));
+  return r;
+}
 // digit at bit offset sh of two half-words as bf16x2 (a low, b high):
 // bf16 0x4300 | d is 128 + d, and s (128 + d) - 128 s = s d exactly
 __device__ __forceinline__ unsigned dig2(unsigned wa, unsigned wb, int sh, unsigned sg, unsigned nb) {
   const unsigned p = ((wa >> sh) & 0x7Fu) | (((wb >> sh) & 0x7Fu) << 16) | 0x43004300u;
-  unsigned r;
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(p), "r"(sg), "r"(nb));
-  return r;
+  return bf16x2_fma(p, sg, nb);
 }
 // a bf16 pair times 2^-7 (exact for the 7-bit digits: no bits are lost)
 __device__ __forceinline__ unsigned bf16x2_scale_m7(unsigned x) {
@@ -338,10 +342,16 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 __device__ __forceinline__ void mbar_init(unsigned long long* mb, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mb)), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(unsigned long long* mb) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(mb)) : "memory");
+}
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long* mb, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mb)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long* mb, unsigned count) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mb)), "r"(count) : "memory");
 }
 // bytes and both addresses multiples of 16
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* mb) {
@@ -359,6 +369,83 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* mb, unsigned p
       : "memory");
   return ok != 0;
 }
+// ------------------------------------------- tcgen05 (5th-generation tensor cores)
+// Tensor memory: 128 lanes x 512 columns of 32 bits per SM; one warp
+// allocates and frees it (column counts are powers of two).
+constexpr unsigned TMEM_COLS = 512;
+__device__ __forceinline__ void tmem_alloc(unsigned* s_base) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_base)),
+               "r"(TMEM_COLS)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(unsigned base) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(TMEM_COLS) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// Shared-memory operand without swizzle: 8 x 8 bf16 blocks (8 rows of 16
+// bytes, 128 bytes in a row), lbo and sbo bytes between blocks.  K-major
+// operands (16 bytes run along K): lbo between blocks along K, sbo along
+// M/N.  M/N-major ones (16 bytes run along M/N): lbo along K, sbo along M/N.
+__device__ __forceinline__ unsigned long long umma_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
+  return (unsigned long long)((saddr >> 4) & 0x3FFFu) | ((unsigned long long)(lbo >> 4) << 16) |
+         ((unsigned long long)(sbo >> 4) << 32) | (1ull << 46);
+}
+// bf16 x bf16 -> FP32, M = 128, N columns, K = 16; a_mn: A is M-major
+__device__ __forceinline__ unsigned umma_idesc(int N, bool a_mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | ((unsigned)(N >> 3) << 17) | (8u << 24);
+}
+// d (+)= a b, issued by one thread; acc = 0 overwrites d
+__device__ __forceinline__ void umma_bf16(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc,
+                                          unsigned acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// True in one thread of warp w (w uniform).  The warp number goes through a
+// shuffle so that the branch is warp-uniform and the elected thread's code
+// keeps descriptors in uniform registers: with a plain threadIdx.x == 0 an
+// MMA took 168 cycles to issue, this way 39 to 64 (its own time).
+__device__ __forceinline__ bool mma_thread(int w = 0) {
+  if (__shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) != w) return false;
+  unsigned el;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(el));
+  return el != 0;
+}
+// arrival on mb when every MMA this thread issued so far is complete
+__device__ __forceinline__ void umma_commit(unsigned long long* mb) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mb))
+               : "memory");
+}
+// N consecutive columns of the warp's 32 lanes (lane quadrant warp % 4)
+template <int N>
+__device__ __forceinline__ void tmem_ld(float* v, unsigned addr) {
+  static_assert(N == 2 || N == 4 || N == 8 || N == 16, "");
+  unsigned r[N];
+  if constexpr (N == 2)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+  else if constexpr (N == 4)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+  else if constexpr (N == 8)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+  else
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+#pragma unroll
+  for (int i = 0; i < N; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
 // 2^e as a double, e in the normal range [-1022, 1023]
 __device__ __forceinline__ double pow2n(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 // x 2^e for |e| <= 2044 by one or two exact power-of-two multiplications

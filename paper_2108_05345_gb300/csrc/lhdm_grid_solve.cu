@@ -8,5 +8,9 @@ __global__ void __launch_bounds__(NT, 1) lhdm_solve_grid_kernel(Inst I, unsigned
   extern __shared__ double dyn[];
   GridTeam tm{(int)blockIdx.x, (int)gridDim.x, bar, err, I.wait_ns, I.bar_extra};
   Engine<GridTeam> e(tm, I, dyn);
+  const TcState tc = tc_open();
+  e.mbs = tc.mbs;
+  e.tmem = tc.tmem;
   e.run();
+  tc_close(tc);
 }

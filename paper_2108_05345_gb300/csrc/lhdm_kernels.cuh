@@ -83,7 +83,7 @@ inline ScratchLayout make_layout(int max_m, int max_n, int team) {
   L.pipelined = team > 1;
   L.Dinv = take(L.pipelined ? nbk * TB * TB : 1);
   L.accb = take(L.pipelined ? nbk * TB : 1);
-  L.Vd = take((size_t)ND * m * 8);  // m x ND x 16 words
+  L.Vd = take((size_t)(m + 32) * ND * KM / 4);  // whole row groups, ND x KM bf16 per row
   L.dtotal = o;
   o = 0;
   L.pos = take(n);
@@ -94,7 +94,7 @@ inline ScratchLayout make_layout(int max_m, int max_n, int team) {
   L.ctl = take(16);
   L.qlist = take(cap);
   L.tflag = take(L.pipelined ? nbk * (1 + TB / SLAB + INV_PARTS) : 1);
-  L.Ver = take(m);
+  L.Ver = take(m + 32);
   L.csign = take(n);
   L.itotal = o;
   return L;
@@ -139,6 +139,44 @@ inline __host__ __device__ void bind_scratch(Inst& I, const ScratchLayout& L, do
   I.wait_ns = WAIT_NS;
   I.bar_extra = 0;
   I.guard_force = 0;
+}
+
+// CTA barriers and tensor memory of the tensor-core commit (every thread of
+// the CTA, once per kernel; the memory is freed by tc_close).
+struct TcState {
+  unsigned long long* mbs;
+  unsigned tmem;
+};
+inline __device__ void tc_barriers(unsigned long long* mb) {
+  if (threadIdx.x == 0) {
+    // V tiles and MMA completions: one arrival; pass-1 slots: C digits worth
+    // 8 and V's copy; accumulator reads: one per warp
+    for (int i = 0; i < 17; ++i) mbar_init(mb + i, i < 5 ? 1 : i < 10 ? 9 : i < 15 ? 1 : NW);
+    fence_mbar_init();
+  }
+}
+inline __device__ TcState tc_open() {
+  __shared__ unsigned long long s_mb[17];
+  __shared__ unsigned s_tmem;
+  if (threadIdx.x < 32) tmem_alloc(&s_tmem);
+  tc_barriers(s_mb);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  return TcState{s_mb, s_tmem};
+}
+// after a wait ran out: fresh barriers for the CTA's next instance
+inline __device__ void tc_reset(const TcState& t) {
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int i = 0; i < 17; ++i) mbar_inval(t.mbs + i);
+  tc_barriers(t.mbs);
+  __syncthreads();
+}
+inline __device__ void tc_close(const TcState& t) {
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x < 32) tmem_free(t.tmem);
 }
 
 inline __device__ void bind_item(Inst& I, const BatchItem& it) {

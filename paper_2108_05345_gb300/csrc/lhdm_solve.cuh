@@ -7,7 +7,7 @@
 namespace lhdm {
 
 // Dynamic shared memory per CTA (bytes) used by the phases below.
-constexpr int DYN_SMEM = 160 * 1024;
+constexpr int DYN_SMEM = 164 * 1024;
 constexpr int CAND_LOCAL_MAX = 2048;     // local DM candidates per CTA
 constexpr int CAND_STAGE = 4096;         // merged candidates staged per pass
 constexpr int ROT_STAGE = 2048;          // rotations staged per pass
@@ -37,6 +37,12 @@ struct Engine {
   int nonfinite = 0;
   bool failed = false;
   bool vd_ok = false;  // the current panel's reflector digits are in Vd/Ver
+  int kdig = 16;       // reflectors their layout holds (the panel's, padded to 16)
+  // tensor-core commit: CTA barriers (MB_*), the parities of their current
+  // phases, tensor memory (set by the kernel)
+  unsigned long long* mbs = nullptr;
+  unsigned mpar = 0u, tmem = 0u;
+  bool tc_failed = false;  // a wait of the tensor-core commit ran out
   int kdm = 0, removed = 0, inner_step = 0;
   int inv_valid = 0;  // positions whose diagonal-block inverse column is current
   int tepoch = 0;     // pipelined-solve calls in this launch (flag values)
@@ -652,46 +658,61 @@ struct Engine {
     kk = i;  // reflectors formed (truncated by the rank bound)
     if constexpr (std::is_same<Team, CtaTeam>::value) {
       // a one-CTA team holds every row: the digits of the tensor-core commit
-      if (I.Vd != nullptr && kk > 4 && kk <= 32) {
+      if (I.Vd != nullptr && kk > 4) {
         __syncthreads();
+        kdig = (kk + 15) & ~15;
+        const int t2 = lane + 32;
+        const double v0a = (lane < kk) ? ldcg(I.vtop + lane) : 1.0, v0b = (t2 < kk) ? ldcg(I.vtop + t2) : 1.0;
         for (int rr = warp; rr < L; rr += NW) {
-          const double v0 = (lane < kk) ? ldcg(I.vtop + lane) : 1.0;
-          const double vr = (lane < kk) ? (rr > lane ? ldcg(V + (size_t)rr * KM + lane) : (rr == lane ? v0 : 0.0)) : 0.0;
-          vd_store_row(rr, vr, v0);
+          const double va = (lane < kk) ? (rr > lane ? ldcg(V + (size_t)rr * KM + lane) : (rr == lane ? v0a : 0.0)) : 0.0;
+          const double vb = (t2 < kk) ? (rr > t2 ? ldcg(V + (size_t)rr * KM + t2) : (rr == t2 ? v0b : 0.0)) : 0.0;
+          vd_store_row(rr, va, v0a, vb, v0b);
         }
+        vd_store_tail(L);
         vd_ok = true;
       }
     }
     return sync();
   }
 
-  // One row of the panel's reflectors as 7-bit digits for the tensor-core
-  // commit (one warp; lane t holds V(row, t) - v0 on the diagonal, zero
-  // above - and v0 of reflector t).  Reflector t is scaled by 2^-Ft,
-  // 2^Ft > |v0| >= |V(:, t)|; the row scale is the largest exponent bound of
-  // the scaled row, and even lanes store digit pairs.
-  __device__ __forceinline__ void vd_store_row(int row, double vrow, double v0) {
-    const double v = scale2(vrow, -ebound(v0));
-    const int er = __reduce_max_sync(0xffffffffu, ebound(v));
-    unsigned ha, la;
-    halves28(fix56(v, 56 - er), ha, la);
-    const unsigned hb = __shfl_down_sync(0xffffffffu, ha, 1), lb = __shfl_down_sync(0xffffffffu, la, 1);
-    const bool nega = v < 0.0;
-    const bool negb = __shfl_down_sync(0xffffffffu, nega ? 1 : 0, 1) != 0;
-    unsigned sg, nb2;
-    sign2(nega, negb, sg, nb2);
-    if ((lane & 1) == 0) {
-      // a row holds its ND digit planes (16 words each) side by side;
-      // 16-byte chunk c of the row is stored at c ^ (row & 7), as the
-      // commit's shared-memory layout expects
-      const int w = lane >> 1;
+  // Row r of the panel's reflectors as 7-bit digits for the tensor-core
+  // commit (one warp; lane t holds V(r, t) and V(r, t + 32) - v0 on the
+  // diagonal, zero above - and v0 of these reflectors, 1 past the panel).
+  // Reflector t is scaled by 2^-Ft, 2^Ft > |v0| >= |V(:, t)|; the row scale
+  // is the largest exponent bound of the scaled row; even lanes store digit
+  // pairs.  Rows go in groups of 8 by their row of W (nP + r), which the
+  // commit's C digits follow; a group holds kdig / 8 blocks of 8 reflectors
+  // per digit, a block 8 rows of 16 bytes (the tensor cores' operand block
+  // without swizzle, for both orientations the commit uses).
+  __device__ __forceinline__ void vd_store_row(int r, double va, double v0a, double vb, double v0b) {
+    const double sa = scale2(va, -ebound(v0a)), sb = scale2(vb, -ebound(v0b));
+    const int er = __reduce_max_sync(0xffffffffu, max(ebound(sa), ebound(sb)));
+    const int row = nP + r, rg = (row >> 3) - (nP >> 3);
 #pragma unroll
-      for (int k = 0; k < ND; ++k) {
-        const int c = (4 * k + (w >> 2)) ^ (row & 7);
-        I.Vd[(size_t)row * (16 * ND) + c * 4 + (w & 3)] = dig2k(k, ha, la, hb, lb, sg, nb2);
+    for (int h = 0; h < 2; ++h) {
+      if (h == 1 && kdig <= 32) break;
+      const double v = h ? sb : sa;
+      unsigned ha, la;
+      halves28(fix56(v, 56 - er), ha, la);
+      const unsigned hb = __shfl_down_sync(0xffffffffu, ha, 1), lb = __shfl_down_sync(0xffffffffu, la, 1);
+      const bool nega = v < 0.0;
+      const bool negb = __shfl_down_sync(0xffffffffu, nega ? 1 : 0, 1) != 0;
+      unsigned sg, nb2;
+      sign2(nega, negb, sg, nb2);
+      const int t = lane + 32 * h, q = kdig >> 3;
+      if ((lane & 1) == 0 && t < kdig) {
+        unsigned* p = I.Vd + ((size_t)rg * ND * q + (t >> 3)) * 32 + (row & 7) * 4 + ((t & 7) >> 1);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) p[k * q * 32] = dig2k(k, ha, la, hb, lb, sg, nb2);
       }
     }
-    if (lane == 0) I.Ver[row] = er;
+    if (lane == 0 && r < I.m - nP) I.Ver[r + (nP & 7)] = er;
+  }
+  // Zero digits for the rows past the last one, to the end of the group
+  // after its own (the commit reads whole pairs of groups).
+  __device__ __forceinline__ void vd_store_tail(int L) {
+    const int end = ((((nP + L - 1) >> 3) + 2) << 3) - nP;
+    for (int r = L + warp; r < end; r += NW) vd_store_row(r, 0.0, 1.0, 0.0, 1.0);
   }
 
   // Panel with the team's rows held in shared memory (at most PR_MAX rows
@@ -720,7 +741,8 @@ struct Engine {
     if (tm.rank == 0)
       for (int e = tid; e < PACC_W; e += NT) I.pacc[e] = 0;
     kk = ldcg(I.ctl + C_KK);
-    vd_ok = I.Vd != nullptr && kk > 4 && kk <= 32;
+    vd_ok = I.Vd != nullptr && kk > 4;
+    kdig = (kk + 15) & ~15;
     return true;
   }
   // The panel on ranks 0 .. P-1 (rows split over them), with the sub-team
@@ -1062,12 +1084,16 @@ struct Engine {
       I.V[(size_t)(q0 + rr) * KM + t] = sP[rr * PS + t];
     }
     // the same rows as 7-bit digits for the tensor-core commit
-    if (I.Vd != nullptr && kk > 4 && kk <= 32) {
+    if (I.Vd != nullptr && kk > 4) {
+      kdig = (kk + 15) & ~15;
+      const int t2 = lane + 32;
+      const double v0a = (lane < kk) ? s_v0[lane] : 1.0, v0b = (t2 < kk) ? s_v0[t2] : 1.0;
       for (int rr = warp; rr < nr; rr += NW) {
         const int row = q0 + rr;
-        vd_store_row(row, (lane < kk) ? (row > lane ? sP[rr * PS + lane] : (row == lane ? s_v0[lane] : 0.0)) : 0.0,
-                     (lane < kk) ? s_v0[lane] : 1.0);
+        vd_store_row(row, (lane < kk) ? (row > lane ? sP[rr * PS + lane] : (row == lane ? v0a : 0.0)) : 0.0, v0a,
+                     (t2 < kk) ? (row > t2 ? sP[rr * PS + t2] : (row == t2 ? v0b : 0.0)) : 0.0, v0b);
       }
+      if (tm.rank == P - 1) vd_store_tail(L);
     }
     if (tm.rank == 0) {
       // T is the inverse of the upper triangle M with M[r][r] = 1/beta_r and
@@ -1692,15 +1718,13 @@ struct Engine {
     return s_nl;
   }
 
-  // Shared-memory layout and chunk sizes of one commit (see commit()).
+  // Operands of one tensor-core commit batch (see commit()).
   struct CommitShape {
-    int L, RC1, RC2, VS;
-    double* wk;        // work area
+    int L;
     double* s_D;       // KM x CB
     double* s_E;       // KM x CB
     const double* s_T; // packed T^T rows
     const double* s_vt;
-    double* s_nrm;     // NW x CB
     const int* s_cid;  // batch columns (-1: b)
   };
   static constexpr int CB = 16;  // Z columns per commit batch
@@ -1710,183 +1734,247 @@ struct Engine {
     return (id >= 0 ? Wcol(id) : I.bt) + nP;
   }
 
-  // Rows [rb, rb+nr) of V (kp columns) into wk with row stride VS.
-  __device__ __forceinline__ void stage_vrows(const CommitShape& cs, int rb, int nr) {
-    const int tot = nr * kp;
-    for (int e0 = tid; e0 < tot; e0 += 4 * NT) {
-      double v[4];
+  // Rows [rb, rb+nr) of V (kp columns, v0 on the diagonal, zero above) into
+  // sV with row stride VS: a warp per row.
+  __device__ __forceinline__ void stage_vrows(double* sV, int VS, const double* s_vt, int rb, int nr) {
+    for (int rr = warp; rr < nr; rr += NW) {
+      const int rg = rb + rr;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int e = e0 + k * NT, rr = e / kp, t = e - rr * kp, rg = rb + rr;
-        v[k] = (e < tot && rg > t) ? ldcg(I.V + (size_t)rg * KM + t) : ((e < tot && rg == t) ? cs.s_vt[t] : 0.0);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int e = e0 + k * NT, rr = e / kp, t = e - rr * kp;
-        if (e < tot) cs.wk[rr * cs.VS + t] = v[k];
+      for (int h = 0; h < 2; ++h) {
+        const int t = lane + 32 * h;
+        if (t < kp) sV[rr * VS + t] = (rg > t) ? ldcg(I.V + (size_t)rg * KM + t) : (rg == t) ? s_vt[t] : 0.0;
       }
     }
   }
 
-  // One batch of NB columns: D = V^T C (pass 1: thread (t1, g1) sums rows
-  // g1, g1+G, ... of every chunk, then a fixed pairwise tree over g1),
-  // D' = T^T D, C -= V D' and the trailing norms (pass 2: thread (r2, grp)
-  // updates row r2 of every chunk in columns grp, grp+NG, ...).  NB is a
-  // template parameter so that no issue slot goes to absent columns.
-  template <int NB>
-  __device__ void commit_batch(const CommitShape& cs) {
-    const int L = cs.L, RC1 = cs.RC1, RC2 = cs.RC2, VS = cs.VS;
-    double* wk = cs.wk;
-    const int G = NT / kp, t1 = tid % kp, g1 = tid / kp;
-    const bool act1 = g1 < G;
-    double acc[NB];
+  // FP64 commit of n columns, 32 at a time with a lane per column: D = V^T C
+  // (a warp per reflector), D' = T^T D, C -= V D' and the trailing norms (a
+  // warp per row).  V and the columns' rows are staged in shared memory, all
+  // of them when they fit, else RC at a time; the next 32 columns are copied
+  // meanwhile when a second buffer fits.  Every operand of an FMA is a
+  // broadcast or 32 consecutive doubles, so it runs at the FP64 pipe's rate:
+  // about kp L 32 cycles per 32 columns (two lane FMAs a cycle) and 4000
+  // beside them.  Every sum runs in an order fixed by kp and L.
+  __device__ void commit_cols(const double* s_T, const double* s_vt, const int* list, int n, int L) {
+    constexpr int XS = 33;
+    const int VS = kp | 1;
+    double* sD = dyn;                    // kp x XS, then D'
+    double* sE = sD + kp * XS;
+    double* sN = sE + kp * XS;           // NW x XS
+    double* wk = sN + NW * XS;
+    const int room = DYN_SMEM / 8 - (2 * kp + NW) * XS;
+    const bool whole = L <= room / (VS + XS);
+    const int RC = whole ? L : (room / (VS + XS)) & ~31;
+    const bool two = whole && L * (VS + 2 * XS) <= room;
+    double* sV = wk;
+    double* sX0 = wk + RC * VS;
+    // rows [rb, rb + nr) of columns base .. into a buffer
+    auto stage_x = [&](double* sX, int base, int rb, int nr) {
+      for (int c = warp; c < 32; c += NW) {
+        const bool in = base + c < n;
+        const int id = in ? list[base + c] : -1;
+        const double* col = (id >= 0 ? Wcol(id) : I.bt) + nP + rb;
+        for (int r = lane; r < nr; r += 32) cp8(sX + r * XS + c, col + r, in);
+      }
+      cp_commit();
+    };
+    __syncthreads();
+    if (whole) stage_vrows(sV, VS, s_vt, 0, L);
+    if (whole) stage_x(sX0, 0, 0, L);
+    for (int base = 0, b = 0; base < n; base += 32, b ^= two ? 1 : 0) {
+      double* sX = sX0 + b * RC * XS;
+      const int nc = min(32, n - base);
+      double acc[4][2];
 #pragma unroll
-    for (int c = 0; c < NB; ++c) acc[c] = 0.0;
-    double* sX = wk + RC1 * VS;  // NB x RC1
-    for (int rb = 0; rb < L; rb += RC1) {
-      const int nr = min(RC1, L - rb);
-      __syncthreads();
-      stage_vrows(cs, rb, nr);
-      const int totx = NB * nr;
-      for (int e0 = tid; e0 < totx; e0 += 4 * NT) {
-        double v[4];
+      for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = 0.0;
+      for (int rb = 0; rb < L; rb += RC) {
+        const int nr = min(RC, L - rb);
+        if (!whole) {
+          __syncthreads();
+          stage_vrows(sV, VS, s_vt, rb, nr);
+          stage_x(sX, base, rb, nr);
+        } else if (!two && base > 0) {
+          stage_x(sX, base, 0, L);
+        }
+        cp_wait_all();
+        __syncthreads();
+        if (two && base + 32 < n) stage_x(sX0 + (b ^ 1) * RC * XS, base + 32, 0, L);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int e = e0 + k * NT, cc = e / nr, rr = e - cc * nr;
-          v[k] = (e < totx) ? ldcg(commit_col(cs.s_cid, cc) + rb + rr) : 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int e = e0 + k * NT, cc = e / nr, rr = e - cc * nr;
-          if (e < totx) sX[cc * RC1 + rr] = v[k];
-        }
-      }
-      __syncthreads();
-      if (act1) {
-        for (int rr = g1; rr < nr; rr += G) {
-          const double v = wk[rr * VS + t1];
-#pragma unroll
-          for (int c = 0; c < NB; ++c) acc[c] = fma(v, sX[c * RC1 + rr], acc[c]);
-        }
-      }
-    }
-    __syncthreads();
-    double* P = wk;  // G x kp x NB partials
-    if (act1) {
-#pragma unroll
-      for (int c = 0; c < NB; ++c) P[(g1 * kp + t1) * NB + c] = acc[c];
-    }
-    __syncthreads();
-    for (int st = 1; st < G; st <<= 1) {
-      if (act1 && (g1 & (2 * st - 1)) == 0 && g1 + st < G) {
-#pragma unroll
-        for (int c = 0; c < NB; ++c) P[(g1 * kp + t1) * NB + c] += P[((g1 + st) * kp + t1) * NB + c];
-      }
-      __syncthreads();
-    }
-    for (int o = tid; o < kp * NB; o += NT) {
-      const int t = o / NB, cc = o - t * NB;
-      cs.s_D[t * CB + cc] = P[t * NB + cc];
-    }
-    __syncthreads();
-    // D' = T^T D
-    for (int o = tid; o < kp * NB; o += NT) {
-      const int t = o % kp, cc = o / kp;
-      double e2 = 0.0;
-      for (int sidx = 0; sidx <= t; ++sidx) e2 = fma(cs.s_T[t * (t + 1) / 2 + sidx], cs.s_D[sidx * CB + cc], e2);
-      cs.s_E[t * CB + cc] = e2;
-    }
-    // pass 2 (NG = 1 or 2 groups of columns)
-    const int NG = NT / RC2, r2 = tid % RC2, grp = tid / RC2;
-    constexpr int NK2 = (NB + 1) / 2;
-    double nrm[NB];
-#pragma unroll
-    for (int k = 0; k < NB; ++k) nrm[k] = 0.0;
-    for (int rb = 0; rb < L; rb += RC2) {
-      const int nr = min(RC2, L - rb);
-      __syncthreads();
-      stage_vrows(cs, rb, nr);
-      __syncthreads();
-      if (r2 < nr) {
-        const bool below = rb + r2 >= kp;
-        if (NG == 1) {
-          double x[NB];
-#pragma unroll
-          for (int k = 0; k < NB; ++k) x[k] = ldcg(commit_col(cs.s_cid, k) + rb + r2);
-          for (int t = 0; t < kp; ++t) {
-            const double v = wk[r2 * VS + t];
-#pragma unroll
-            for (int k = 0; k < NB; ++k) x[k] = fma(-v, cs.s_E[t * CB + k], x[k]);
+          const int t = warp + k * NW;
+          if (t >= kp) break;
+          // V(r, t) = 0 above row t
+          double a0 = acc[k][0], a1 = acc[k][1];
+          int rr = max(0, t - rb);
+          for (; rr + 3 < nr; rr += 4) {
+            a0 = fma(sV[rr * VS + t], sX[rr * XS + lane], a0);
+            a1 = fma(sV[(rr + 1) * VS + t], sX[(rr + 1) * XS + lane], a1);
+            a0 = fma(sV[(rr + 2) * VS + t], sX[(rr + 2) * XS + lane], a0);
+            a1 = fma(sV[(rr + 3) * VS + t], sX[(rr + 3) * XS + lane], a1);
           }
-#pragma unroll
-          for (int k = 0; k < NB; ++k) {
-            commit_col(cs.s_cid, k)[rb + r2] = x[k];
-            if (below) nrm[k] = fma(x[k], x[k], nrm[k]);
-          }
-        } else {
-          double x[NK2];
-#pragma unroll
-          for (int k = 0; k < NK2; ++k) {
-            const int c = grp + 2 * k;
-            x[k] = (c < NB) ? ldcg(commit_col(cs.s_cid, c) + rb + r2) : 0.0;
-          }
-          for (int t = 0; t < kp; ++t) {
-            const double v = wk[r2 * VS + t];
-#pragma unroll
-            for (int k = 0; k < NK2; ++k) {
-              const int c = grp + 2 * k;
-              if (c < NB) x[k] = fma(-v, cs.s_E[t * CB + c], x[k]);
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < NK2; ++k) {
-            const int c = grp + 2 * k;
-            if (c < NB) {
-              commit_col(cs.s_cid, c)[rb + r2] = x[k];
-              if (below) nrm[k] = fma(x[k], x[k], nrm[k]);
-            }
-          }
+          for (; rr < nr; ++rr) a0 = fma(sV[rr * VS + t], sX[rr * XS + lane], a0);
+          acc[k][0] = a0;
+          acc[k][1] = a1;
         }
       }
-    }
-    // norms: a group's threads are whole warps; column c = grp + NG k
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      const int c = grp + NG * k;
-      if (c < NB) {
-        const double v = warp_sum(nrm[k]);
-        if (lane == 0) cs.s_nrm[warp * CB + c] = v;
+      for (int k = 0; k < 4; ++k) {
+        const int t = warp + k * NW;
+        if (t < kp) sD[t * XS + lane] = acc[k][0] + acc[k][1];
+      }
+      __syncthreads();
+      for (int t = warp; t < kp; t += NW) {
+        const double* tr = s_T + t * (t + 1) / 2;
+        double e0 = 0.0, e1 = 0.0;
+        int q = 0;
+        for (; q + 1 <= t; q += 2) {
+          e0 = fma(tr[q], sD[q * XS + lane], e0);
+          e1 = fma(tr[q + 1], sD[(q + 1) * XS + lane], e1);
+        }
+        if (q <= t) e0 = fma(tr[q], sD[q * XS + lane], e0);
+        sE[t * XS + lane] = e0 + e1;
+      }
+      double nrm = 0.0;
+      for (int rb = 0; rb < L; rb += RC) {
+        const int nr = min(RC, L - rb);
+        if (!whole) {
+          __syncthreads();
+          stage_vrows(sV, VS, s_vt, rb, nr);
+          stage_x(sX, base, rb, nr);
+          cp_wait_all();
+        }
+        __syncthreads();
+        for (int rr = warp; rr < nr; rr += NW) {
+          const int te = min(rb + rr + 1, kp);
+          double x0 = sX[rr * XS + lane], x1 = 0.0;
+          const double* v = sV + rr * VS;
+          int t = 0;
+          for (; t + 3 < te; t += 4) {
+            x0 = fma(-v[t], sE[t * XS + lane], x0);
+            x1 = fma(-v[t + 1], sE[(t + 1) * XS + lane], x1);
+            x0 = fma(-v[t + 2], sE[(t + 2) * XS + lane], x0);
+            x1 = fma(-v[t + 3], sE[(t + 3) * XS + lane], x1);
+          }
+          for (; t < te; ++t) x0 = fma(-v[t], sE[t * XS + lane], x0);
+          x0 += x1;
+          sX[rr * XS + lane] = x0;
+          if (rb + rr >= kp) nrm = fma(x0, x0, nrm);
+        }
+        __syncthreads();
+        for (int c = warp; c < nc; c += NW) {
+          const int id = list[base + c];
+          double* col = (id >= 0 ? Wcol(id) : I.bt) + nP + rb;
+          for (int r = lane; r < nr; r += 32) col[r] = sX[r * XS + c];
+        }
+      }
+      sN[warp * XS + lane] = nrm;
+      __syncthreads();
+      if (warp == 0 && lane < nc) {
+        double v = 0.0;
+        for (int w = 0; w < NW; ++w) v += sN[w * XS + lane];
+        const int id = list[base + lane];
+        if (id >= 0) I.u[id] = sqrt(v);
       }
     }
+  }
+
+  // FP64 commit of n <= 8 columns (a CTA's share when the team has more CTAs
+  // than a few columns each) with V and the columns in shared memory: a warp
+  // per (reflector, column) dot, then four or two warps per column for the
+  // update, lanes over the rows.  L (kp + 1 + n) doubles must fit.
+  __device__ void commit_narrow(const double* s_T, const double* s_vt, const int* list, int n, int L) {
+    const int VS = kp | 1;
+    double* sD = dyn;                 // kp x 8, then D'
+    double* sE = sD + KM * 8;
+    double* sN = sE + KM * 8;         // NW
+    double* sV = sN + 32;
+    double* sX = sV + L * VS;         // n x L
     __syncthreads();
-    if (tid < NB) {
-      const int g = tid % NG, w0 = g * (RC2 / 32);
+    for (int c = warp & 7; c < n; c += 8) {
+      const int id = list[c];
+      const double* col = (id >= 0 ? Wcol(id) : I.bt) + nP;
+      for (int r = lane + 32 * (warp >> 3); r < L; r += 64) cp8(sX + c * L + r, col + r, true);
+    }
+    cp_commit();
+    stage_vrows(sV, VS, s_vt, 0, L);
+    cp_wait_all();
+    __syncthreads();
+    for (int o = warp; o < kp * n; o += NW) {
+      const int t = o / n, c = o - t * n;
+      double a0 = 0.0, a1 = 0.0;
+      int r = (t & ~31) + lane;  // V(r, t) = 0 above row t
+      for (; r + 32 < L; r += 64) {
+        a0 = fma(sV[r * VS + t], sX[c * L + r], a0);
+        a1 = fma(sV[(r + 32) * VS + t], sX[c * L + r + 32], a1);
+      }
+      if (r < L) a0 = fma(sV[r * VS + t], sX[c * L + r], a0);
+      const double v = warp_sum(a0 + a1);
+      if (lane == 0) sD[t * 8 + c] = v;
+    }
+    __syncthreads();
+    for (int o = tid; o < kp * 8; o += NT) {
+      const int t = o >> 3, c = o & 7;
+      const double* tr = s_T + t * (t + 1) / 2;
+      double e = 0.0;
+      if (c < n)
+        for (int q = 0; q <= t; ++q) e = fma(tr[q], sD[q * 8 + c], e);
+      sE[o] = e;
+    }
+    __syncthreads();
+    const int wc = n <= 4 ? 4 : 8, c = warp & (wc - 1), part = warp / wc, np = NW / wc;  // np warps per column
+    double nrm = 0.0;
+    if (c < n) {
+      const int id = list[c];
+      double* col = (id >= 0 ? Wcol(id) : I.bt) + nP;
+      for (int r = lane + 32 * part; r < L; r += 32 * np) {
+        double x0 = sX[c * L + r], x1 = 0.0;
+        const double* v = sV + r * VS;  // zero above the diagonal
+        int t = 0;
+        for (; t + 1 < kp; t += 2) {
+          x0 = fma(-v[t], sE[t * 8 + c], x0);
+          x1 = fma(-v[t + 1], sE[(t + 1) * 8 + c], x1);
+        }
+        if (t < kp) x0 = fma(-v[t], sE[t * 8 + c], x0);
+        x0 += x1;
+        col[r] = x0;
+        if (r >= kp) nrm = fma(x0, x0, nrm);
+      }
+    }
+    nrm = warp_sum(nrm);
+    if (lane == 0) sN[warp] = nrm;
+    __syncthreads();
+    if (tid < n) {
       double v = 0.0;
-      for (int w2 = 0; w2 < RC2 / 32; ++w2) v += cs.s_nrm[(w0 + w2) * CB + tid];
-      if (cs.s_cid[tid] >= 0) I.u[cs.s_cid[tid]] = sqrt(v);
+      for (int w = 0; w < np; ++w) v += sN[w * wc + tid];
+      if (list[tid] >= 0) I.u[list[tid]] = sqrt(v);
     }
+    __syncthreads();
   }
 
-  // One batch of nb <= NBP (8 or 16) columns through the bf16 tensor cores,
-  // for 5 <= kp <= 16 KT (KT = 1 or 2 tiles of 16 reflectors) with the
-  // panel's reflector digits in Vd/Ver.
+  // One batch of nb <= NB (8 or 16) columns through the tensor cores, for
+  // 5 <= kp <= KM with the panel's reflector digits in Vd/Ver.  Both passes
+  // are tcgen05.mma (M = 128, FP32 accumulators in tensor memory), issued by
+  // one thread while all warps prepare operands or drain accumulators.
   //  pass 1: D = V^T C.  With V(r, :) = 2^Er v'(r, :) (|v'| < 1, digits a_k
   //    from the panel) and C' = 2^Er C (digits c_l under the column scale
   //    2^Ec), D = 2^(Ec-14) sum_lam 2^(-7 lam) sum_{k+l=lam} a_k^T c_l.
-  //    64-row chunks, double-buffered: the next chunk's V digits arrive by
-  //    cp.async and its C values are loaded while the tensor cores work on
-  //    the current one.  Warp (tile pair, sub) takes rows sub*16 .. +15 of
-  //    every chunk for one 16 x 8 (reflector, column) tile and keeps one
-  //    FP32 accumulator per level k + l <= 8, moved to int32 every 128 of
-  //    its rows (exact: at most 8 pairs of products below 2^14 per row).
+  //    M runs over (digit k, reflector t), N over (digit l, column c), K over
+  //    the rows: every digit pair has its own accumulator, exact for 1024
+  //    rows (127^2 x 1024 < 2^24), then moved into int32 level sums.  The
+  //    M tile that starts at digit k0 takes the column digits l <= 8 - k0
+  //    only.  Chunks of 32 or 64 rows go through a ring of three to five
+  //    slots: V's digits arrive by bulk copies, fourteen warps turn C values
+  //    into digits, one thread issues the MMAs.
   //  D' = T^T D in FP64.
-  //  pass 2: C -= V D'.  128-row chunks, double-buffered.  From the digits
-  //    of V (row scale) and of D'' = 2^Ft D' (column scale 2^Ee) warp (row
-  //    tile, column tile) forms the 9 level sums of its 16 x 8 tile (exact
-  //    in FP32: at most 8 pairs x 32 terms), combines them in int64
-  //    (u = sum_lam lev_lam 2^(43-7 lam), levels 7 and 8 rounded down;
-  //    |u| < 2^63 as lev_lam < (lam+1) 2^19) and applies x -= u 2^(Er+Ee-57)
-  //    and the trailing norm in FP64.
+  //  pass 2: C -= V D'.  128-row tiles: M = rows, K = reflectors.  For V
+  //    digit k one MMA takes the digits l <= 8 - k of D'' = 2^Ft D' (column
+  //    scale 2^Ee) as N = (l, column) and adds into the tensor-memory columns
+  //    that start at k NB, so the accumulators are the nine level sums
+  //    (exact: at most 8 pairs x 64 terms below 2^14).  A thread combines
+  //    them for its row in int64 (u = sum_lam lev_lam 2^(43-7 lam), levels 7
+  //    and 8 rounded down; |u| < 2^63 as lev_lam < (lam+1) 2^20) and applies
+  //    x -= u 2^(Er+Ee-57) and the trailing norm in FP64 while the next
+  //    tile's MMAs run into the other accumulator half.
   //  Reflector scales: V's digits are of V(r, t) / 2^Ft with 2^Ft > |v0_t|
   //    >= |V(:, t)| (the panel scales each reflector by its own power of
   //    two before the row scale is taken), so reflectors of very different
@@ -1894,302 +1982,461 @@ struct Engine {
   //    norm after the earlier reflectors - keep all their digits; the factor
   //    2^Ft returns in D (pass 1) and in D'' (pass 2).
   // Every sum is exact or in a fixed order, so the result is bitwise
-  // reproducible.  Shared memory (bytes of the work area): V digit buffers
-  // [0, 64K) and [64K, 128K) (R rows of 512 B: the ND digit planes side by
-  // side, 16-byte chunks XOR-swizzled by row so that ldmatrix is
-  // conflict-free), pass-1 C' digit buffers in the upper halves of those
-  // (pass 1 has R = 64), D' digits at 128K.
+  // reproducible.  What bounds it: pass 2 the two FP64 operations per
+  // element (2048 cycles per 128 rows x 16 columns at 2 lane-ops/clk/SM;
+  // measured about 2900), pass 1 the issuing thread's waits and MMAs (about
+  // 700 cycles per 32 rows and 32 reflectors), and some 25 000 cycles a batch
+  // in the steps between.  Against the mma.sync form this replaced (5 <= kp
+  // <= 32; FP64 above): commit phase 12.7 -> 6.8 ms at 4096 x 2048, k_max 32;
+  // 5.8 -> 2.1 ms at 2048 x 8192, k_max 64.
   // Accuracy guard of pass 1.  The fixed-point digits carry 56 bits under
   // one power-of-two scale per V row and per column of C', so a sum whose
   // terms all lie far below the scale (a large entry of C paired with zeros
   // of V, say) loses bits that an FP64 dot product would keep.  Pass 1 also
-  // forms the sum of |leading digit| products (one more MMA per step, exact
-  // integers), a lower bound of sum |v'||c'| over the digit rows in units
-  // of 2^(Ec - 14).  The digit result's error is at most 2L 2^(Ec-57) (times
-  // 2^Ft); where that could exceed the worst-case bound of the FP64
+  // bounds from below the sum of |leading digit| products, sum |v'||c'| over
+  // the digit rows in units of 2^(Ec - 14): by |D| itself, by the rows still
+  // in shared memory at its end, and by all rows where those do not suffice.  The digit result's error is at most 2L 2^(Ec-57)
+  // (times 2^Ft); where that could exceed the worst-case bound of the FP64
   // evaluation, gamma_L sum |v||c| - i.e. where the digit rows' sum plus the
   // FP64 rows' sum |v||c| stays below 2^(Ec-3) (2^11 in the digits' units) -
   // the batch goes to the FP64 commit before any column is touched.
   static constexpr float GUARD1 = 2048.0f;  // 2^11: sum |v'||c'| >= 2^(Ec-3)
   static constexpr unsigned ABS2 = 0x7FFF7FFFu;  // clears the signs of a bf16 pair
 
+  // CTA barriers of the tensor-core commit (mbs): V tiles arrived (bulk
+  // copies), a pass-1 slot's V chunk arrived and its C digits written
+  // (arrivals worth 8 per chunk and the copy's), MMAs of a slot complete,
+  // accumulators of a pass-2 half read (one arrival per warp).  mpar holds the parity of each barrier's current phase.
+  enum { MB_V = 0, MB_C = 5, MB_F = 10, MB_T = 15 };
+  // Bounded wait for the phase `ahead` uses after the current one of barrier
+  // i; a thread whose wait ran out does not wait again.
+  __device__ __forceinline__ void mb_wait(int i, int ahead, bool& ok) {
+    if (!ok) return;
+    const unsigned par = ((mpar >> i) ^ (unsigned)ahead) & 1u;
+    if (mbar_try_wait(mbs + i, par)) return;
+    const long long t0 = gtimer();
+    unsigned spins = 0;
+    while (!mbar_try_wait(mbs + i, par)) {
+      if ((++spins & 255u) == 0u && gtimer() - t0 > WAIT_NS) {
+        ok = false;
+        return;
+      }
+    }
+  }
+
+  // Digits l the M tile mt of pass 1 takes (MT = KP / 16 tiles of 128 pairs
+  // (digit k, reflector)): l <= 8 - its first k, N a multiple of 16.
+  template <int NB>
+  __device__ static constexpr int tile_digits(int mt, int MT) {
+    const int n = NLV - 8 * mt / MT, e = (NB == 16) ? n : (n + 1) & ~1;
+    return e < ND ? e : ND;
+  }
+  // Ring of pass 1: row groups per chunk, slots.
+  __device__ static constexpr int p1_groups(int MT) { return MT == 1 ? 8 : 4; }
+  __device__ static constexpr int p1_slots(int MT) { return MT == 2 ? 5 : MT == 4 ? 3 : 4; }
+  // The MMAs of a pass-1 chunk (16 rows per step, nks <= 4 steps) and of a
+  // pass-2 tile; one thread.  Unrolled with constant descriptor steps: the
+  // issuing thread's instructions must fit beside an MMA's 40 to 72 cycles.
+  template <int NB, int MT>
+  __device__ __forceinline__ void issue_pass1(unsigned av, unsigned bv, int nks, unsigned more) {
+    constexpr unsigned RGB = MT * 2048, CGB = ND * (NB / 8) * 128;  // bytes per row group of V, of C digits
+    const unsigned long long da = umma_desc(av, RGB, 128), db = umma_desc(bv, CGB, 128);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      if (ks >= nks) break;
+      unsigned toff = 0;
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        umma_bf16(tmem + toff, da + ((ks * 2 * RGB + mt * 2048) >> 4), db + ((ks * 2 * CGB) >> 4),
+                  umma_idesc(tile_digits<NB>(mt, MT) * NB, true), ks ? 1u : more);
+        toff += tile_digits<NB>(mt, MT) * NB;
+      }
+    }
+  }
+  // n chunks from ring position (slot, use) on, as their operands arrive;
+  // chunk jr has nkr steps.  One thread.
+  template <int NB, int MT>
+  __device__ __forceinline__ void mma_chunks(unsigned av0, unsigned bv0, int slot, int use, int n, int jr, int nkr,
+                                             bool& ok) {
+    constexpr int G1 = p1_groups(MT), NR = p1_slots(MT);
+    constexpr unsigned VB = G1 * MT * 2048, CBB = G1 * ND * (NB / 8) * 128;
+    for (int j = 0; j < n; ++j) {
+      mb_wait(MB_C + slot, use, ok);
+      if (!ok) return;
+      tc_fence_after();
+      issue_pass1<NB, MT>(av0 + slot * VB, bv0 + slot * CBB, j == jr ? nkr : G1 / 2, j ? 1u : 0u);
+      umma_commit(mbs + MB_F + slot);
+      if (++slot == NR) {
+        slot = 0;
+        ++use;
+      }
+    }
+  }
+  template <int NB, int MT>
+  __device__ __forceinline__ void issue_pass2(unsigned av, unsigned bv, unsigned acc0) {
+    constexpr int NPL = NB == 16 ? 9 : 10;
+    constexpr unsigned RGB = MT * 2048, EGB = NPL * (NB / 8) * 128;  // bytes per 8 rows of V, per 8 reflectors of D''
+    const unsigned long long da = umma_desc(av, 128, RGB), db = umma_desc(bv, EGB, 128);
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      // digits l <= 8 - k; k = 0 also clears level 8 (a zero digit plane)
+      const int cnt = (k == 0) ? NPL : (NB == 16) ? NLV - k : (NLV - k + 1) & ~1;
+#pragma unroll
+      for (int ks = 0; ks < MT; ++ks)
+        umma_bf16(acc0 + k * NB, da + ((k * MT * 256 + ks * 256) >> 4), db + ((ks * 2 * EGB) >> 4),
+                  umma_idesc(cnt * NB, false), (k | ks) ? 1u : 0u);
+    }
+  }
+
   // Returns 0 when the batch is committed, 1 when a bounded wait expired, 2
   // when the accuracy guard hands the batch to the FP64 path (C untouched).
-  template <int NBP, int KT>
-  __device__ int commit_tc(const CommitShape& cs, int nb) {
-    constexpr int NTN = NBP / 8;           // column tiles
-    constexpr int COMBOS = KT * NTN;       // (reflector tile, column tile) pairs
-    constexpr int MW = COMBOS * 4;         // pass-1 MMA warps
-    constexpr int R1 = 64, R2 = 128;       // rows per chunk in pass 1 and 2
-    constexpr int BUF = ND * 128 * 32;     // bf16 per V digit buffer
-    constexpr int SB = R1 + 8;             // row stride of C' digits (bf16)
-    constexpr int SE = 40;                 // row stride of D' digits (bf16)
-    const int L = cs.L;
+  template <int NB>
+  __device__ __forceinline__ int commit_tc(const CommitShape& cs, int nb) {
+    constexpr int NG = NB / 8;             // column groups of 8
+    constexpr int NPL = NB == 16 ? 9 : 10; // digit planes of D'' (zero from ND on)
+    const int L = cs.L, KP = kdig;         // reflectors, padded to 16
+    const int MT = KP >> 4;                // M tiles of pass 1
+    const unsigned RGB = KP * 128;         // bytes of a group of 8 digit rows
     // The digits cover rows [r0d, L); the first r0d rows - the reflectors'
     // triangle (pivots and the zeros above them, whose row scales would
-    // outweigh every other row), rounded up to a multiple of 8 so that the
-    // staged digit rows keep the row swizzle of Vd - are done in FP64.
-    // Chunk rows below are counted from row r0d.
-    const int r0d = (kp + 7) & ~7;
+    // outweigh every other row), up to the next row of W that is a multiple
+    // of 8, so that the digit rows are whole groups of 8 and the columns'
+    // rows are aligned pairs - are done in FP64.
+    const int r0d = kp + ((8 - ((nP + kp) & 7)) & 7);
     const int Ld = L - r0d;
-    unsigned short* sV = reinterpret_cast<unsigned short*>(cs.wk);
-    unsigned short* sE = sV + 2 * BUF;
+    const int ngr = (((Ld + 7) >> 3) + 1) & ~1;  // digit row groups, even (the panel zeroes the last ones' tail)
+    const unsigned char* gV = reinterpret_cast<const unsigned char*>(I.Vd) + (size_t)(((nP + r0d) >> 3) - (nP >> 3)) * RGB;
+    const int* ver = I.Ver + r0d + (nP & 7);  // 32-byte aligned, like the columns' rows (16)
     __shared__ int s_Ec[CB], s_Ee[CB];
-    const int g = lane >> 2, tq = lane & 3;
-    // digit k, 16-byte chunk q (reflectors 8q .. 8q+7) of staged row r:
-    // rows of 512 bytes, chunk 4k + q at (4k + q) ^ (r & 7)
-    auto vaddr = [&](const unsigned short* base, int, int k, int r, int q) {
-      return base + r * (16 * ND * 2) + (((4 * k + q) ^ (r & 7)) << 3);
-    };
-    // V digits of rows rb .. rb+R into buffer b: one bulk copy (the rows are
-    // stored pre-swizzled), completing on the buffer's mbarrier; rows past L
-    // are zeroed by the threads.  Every thread orders
-    // its generic writes of the work area before later async copies (proxy
-    // fence at entry, before pass 2 and after zeroing).
-    __shared__ unsigned long long s_mbar[2];
-    unsigned vph = 0u;  // bit b: parity of buffer b's next phase
-    fence_proxy_async();
-    if (tid == 0) {
-      mbar_init(&s_mbar[0], 1);
-      mbar_init(&s_mbar[1], 1);
-      fence_mbar_init();
-    }
-    __syncthreads();
-    auto stage_v = [&](int rb, int R, int b) {
-      unsigned short* dst = sV + b * BUF;
-      const int nr = min(R, Ld - rb);
-      if (tid == 0) {
-        mbar_expect_tx(&s_mbar[b], (unsigned)(nr * 64 * ND));
-        bulk_g2s(dst, I.Vd + (size_t)(r0d + rb) * (16 * ND), (unsigned)(nr * 64 * ND), &s_mbar[b]);
-      }
-      if (nr < R) {
-        for (int e = nr * 4 * ND + tid; e < R * 4 * ND; e += NT)
-          *reinterpret_cast<uint4*>(dst + e * 8) = make_uint4(0u, 0u, 0u, 0u);
-        fence_proxy_async();
-      }
-    };
-    // wait for buffer b's copies (bounded); false on expiry
-    auto wait_v = [&](int b) -> bool {
-      const unsigned par = (vph >> b) & 1u;
-      vph ^= 1u << b;
-      const long long t0 = gtimer();
-      unsigned spins = 0;
-      while (!mbar_try_wait(&s_mbar[b], par)) {
-        if ((++spins & 255u) == 0u && gtimer() - t0 > WAIT_NS) return false;
-      }
-      return true;
-    };
+    __shared__ double* s_cp[CB];  // columns from the first digit row on (absent ones: the first)
+    bool ok = true;
     auto expired = [&]() {
       if (tid == 0) {
         int* er = tm_err();
         if (er) atomicExch(er, 1);
       }
     };
-    // column scales of C' = 2^Er C: (column, row quarter) per warp, 8 rows
-    // per lane in flight
-    if (tid < CB) s_Ec[tid] = -8000;
-    __syncthreads();
-    for (int p = warp; p < nb * 4; p += NW) {
-      const int c = p >> 2;
-      const double* col = commit_col(cs.s_cid, c) + r0d;
-      const int* ver = I.Ver + r0d;
-      int lo, hi;
-      split(Ld, 4, p & 3, lo, hi);
-      int mx = -8000;
-      for (int r0 = lo + lane; r0 < hi; r0 += 256) {
-        double xv[8];
-        int ev[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int r = r0 + 32 * u;
-          xv[u] = (r < hi) ? ldcg(col + r) : 0.0;
-          ev[u] = (r < hi) ? ldcg(ver + r) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int e = ebound(xv[u]);
-          if (e > -2000) mx = max(mx, e + ev[u]);
-        }
-      }
-      mx = __reduce_max_sync(0xffffffffu, mx);
-      if (lane == 0) atomicMax(&s_Ec[c], mx);
+    if (tid < CB) {
+      s_Ec[tid] = -8000;
+      s_cp[tid] = commit_col(cs.s_cid, tid < nb ? tid : 0) + r0d;
     }
+    fence_proxy_async();  // generic writes of the work area before the async copies into it
     __syncthreads();
-    // ---- pass 1
-    const int nch1 = (Ld + R1 - 1) / R1;
-    const bool mw = warp < MW;
-    const int cmb = warp % COMBOS, sub = warp / COMBOS;
-    const int mt = cmb % KT, nt = cmb / KT;
-    // C' digits: thread (column tid/32, row pair tid%32) of each chunk, from
-    // the chunk's C values and row exponents, staged by cp.async in the
-    // buffer's [50K, 58.25K) bytes
-    const bool dw = tid < NBP * 32;
-    const int dc = tid >> 5, drr = 2 * (tid & 31);
-    const int dec = (dw && dc < nb) ? s_Ec[dc] : 0;
-    auto cstage = [&](int b) { return reinterpret_cast<double*>(sV + b * BUF) + 6400; };
-    auto stage_c = [&](int rb, int b) {
-      double* sC = cstage(b);
-      int* sR = reinterpret_cast<int*>(sC + NBP * R1);
-      for (int e = tid; e < NBP * R1; e += NT) {
-        const int c = e / R1, r = e - c * R1;
-        const bool ok = c < nb && rb + r < Ld;
-        cp8(sC + e, ok ? commit_col(cs.s_cid, c) + r0d + rb + r : I.u, ok);
+    // column scales of C' = 2^Er C: a warp takes every NW-th group of 128
+    // rows of all columns, sixteen loads in flight (clamped, not predicated:
+    // a branch per load kept them apart and cost 470 cycles each)
+    for (int rb = warp * 128; rb < Ld; rb += NW * 128) {
+      int ev[4], rr[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        rr[u] = min(rb + 32 * u + lane, Ld - 1);
+        ev[u] = ldcg(ver + rr[u]);
       }
-      if (tid < R1) cp4(sR + tid, rb + tid < Ld ? I.Ver + r0d + rb + tid : I.Ver, rb + tid < Ld);
-      cp_commit();
-    };
-    auto digits_c = [&](int b) {
-      if (!dw) return;
-      const double* sC = cstage(b);
-      const int* sR = reinterpret_cast<const int*>(sC + NBP * R1);
-      const double xa = sC[dc * R1 + drr], xb = sC[dc * R1 + drr + 1];
-      unsigned short* sBb = sV + b * BUF + BUF / 2;
-      unsigned ha, la, hb, lb, sg, nb2;
-      halves28(fix56(xa, sR[drr] + 56 - dec), ha, la);
-      halves28(fix56(xb, sR[drr + 1] + 56 - dec), hb, lb);
-      sign2(xa < 0.0, xb < 0.0, sg, nb2);
+      for (int c0 = 0; c0 < nb; c0 += 4) {
+        double xv[4][4];
 #pragma unroll
-      for (int k = 0; k < ND; ++k) *reinterpret_cast<unsigned*>(sBb + (k * NBP + dc) * SB + drr) = dig2k(k, ha, la, hb, lb, sg, nb2);
-    };
-    // levels 0 .. NEX-1 move every 128 rows into exact int32 sums in shared
-    // memory (shared atomics: exact, so the order of the warps does not
-    // matter); levels NEX .. 8 stay in FP32, where their rounding weighs
-    // below 2^-54 of the scales
-    constexpr int NEX = 7;
-    int* sF = reinterpret_cast<int*>(reinterpret_cast<char*>(sV) + 131072);  // COMBOS x NEX x 32 x 4
-    for (int e = tid; e < COMBOS * NEX * 128; e += NT) sF[e] = 0;
-    float acc[NLV][4];
+        for (int j = 0; j < 4; ++j) {
+          const double* col = s_cp[c0 + j];
 #pragma unroll
-    for (int l = 0; l < NLV; ++l)
+          for (int u = 0; u < 4; ++u) xv[j][u] = ldcg(col + rr[u]);
+        }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[l][j] = 0.f;
-    float gacc[4] = {0.f, 0.f, 0.f, 0.f};  // sum of |leading digit| products (guard)
-    int since = 0;
+        for (int j = 0; j < 4; ++j) {
+          int mx = -8000;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int e = ebound(xv[j][u]);
+            mx = max(mx, e > -2000 ? e + ev[u] : -8000);
+          }
+          mx = __reduce_max_sync(0xffffffffu, mx);
+          if (lane == 0) atomicMax(&s_Ec[c0 + j], mx);
+        }
+      }
+    }
+    // ---- pass 1
+    // Warp 0 issues the MMAs, warp 1 the bulk copies of V's digits, the
+    // others turn C into digits: a warp takes 16 rows x 8 columns at a time
+    // (four values a lane).  NR slots hold a chunk of V digits and one of C
+    // digits each.
+    const int G1 = p1_groups(MT), NR = p1_slots(MT);
+    const int nch = (ngr + G1 - 1) / G1;
+    unsigned char* base = reinterpret_cast<unsigned char*>(dyn);
+    int* sF = reinterpret_cast<int*>(base + KM * CB * 8);  // level sums: [lam][reflector][column ^ reflector]
+    unsigned char* sV = base + KM * CB * 8 + NLV * NB * KP * 4;
+    unsigned char* sC = sV + NR * G1 * RGB;                // [row group][digit][column group] blocks
+    const unsigned CBB = G1 * ND * NG * 128;               // bytes of a C digit chunk
+    for (int e = tid; e < NLV * NB * KP; e += NT) sF[e] = 0;
     // every CTA walks the chunks from its own starting chunk, so that the
     // CTAs do not all ask for the same digit rows at the same moment (the
     // sums are exact, so the order does not matter)
-    const int s1 = tm.rank % nch1;
-    auto row1 = [&](int jc) { return ((jc + s1) % nch1) * R1; };
-    stage_c(row1(0), 0);
-    stage_v(row1(0), R1, 0);
-    cp_wait_all();
-    __syncthreads();
-    digits_c(0);
-    for (int jc = 0; jc < nch1; ++jc) {
-      const int b = jc & 1;
-      const bool okv = wait_v(b);
-      if (__syncthreads_or(!okv)) {
+    const int s1 = tm.rank % nch;
+    auto chunk = [&](int j) { const int c = j + s1; return c >= nch ? c - nch : c; };
+    auto groups = [&](int j) { return min(G1, ngr - chunk(j) * G1); };  // even
+    // the accumulators of the finished chunks into the level sums
+    auto flush = [&]() {
+      tc_fence_after();
+      int toff = 0;
+      for (int j = 0; j < MT; ++j) {
+        const int nl = tile_digits<NB>(j, MT);
+        const int mi = 128 * j + 32 * (warp & 3) + lane, k = mi / KP, t = mi - k * KP;
+        for (int l = warp >> 2; l < nl; l += 4) {
+          float v[NB];
+          tmem_ld<NB>(v, tmem + ((unsigned)(32 * (warp & 3)) << 16) + toff + l * NB);
+          tmem_ld_wait();
+          if (k + l < NLV && t < kp) {
+#pragma unroll
+            for (int c = 0; c < NB; ++c)
+              if (c < nb) atomicAdd(sF + ((k + l) * KP + t) * NB + (c ^ (t & (NB - 1))), __float2int_rn(v[c]));
+          }
+        }
+        toff += nl * NB;
+      }
+      tc_fence_before();
+    };
+    const int SEG = 128 / G1;  // chunks per exact accumulation (1024 rows)
+    __syncthreads();            // s_Ec, sF
+    // slot and use (chunk j: slot j mod NR, use j / NR) of this warp's next
+    // chunk, kept by counting (a division is as long as a chunk's MMAs)
+    int slot = 0, use = 0;
+    for (int j0 = 0; j0 < nch; j0 += SEG) {
+      const int j1 = min(nch, j0 + SEG);
+      const int slot0 = slot, use0 = use;  // of chunk j0
+      if (warp == 0) {
+        if (mma_thread()) {
+          // the ragged chunk (the last one of the rows) and its steps
+          const int jr = nch - 1 - s1 - j0;
+          const int nkr = (ngr - (nch - 1) * G1) >> 1;
+          switch (MT) {
+            case 1: mma_chunks<NB, 1>(smem_u32(sV), smem_u32(sC), slot, use, j1 - j0, jr, nkr, ok); break;
+            case 2: mma_chunks<NB, 2>(smem_u32(sV), smem_u32(sC), slot, use, j1 - j0, jr, nkr, ok); break;
+            case 3: mma_chunks<NB, 3>(smem_u32(sV), smem_u32(sC), slot, use, j1 - j0, jr, nkr, ok); break;
+            default: mma_chunks<NB, 4>(smem_u32(sV), smem_u32(sC), slot, use, j1 - j0, jr, nkr, ok); break;
+          }
+        }
+        __syncwarp();
+      } else if (warp == 1) {
+        if (lane == 0) {
+          for (int j = j0; j < j1; ++j) {
+            if (j >= NR) mb_wait(MB_F + slot, use - 1, ok);
+            if (!ok) break;
+            const unsigned bytes = (unsigned)groups(j) * RGB;
+            mbar_expect_tx(mbs + MB_C + slot, bytes);
+            bulk_g2s(sV + slot * G1 * RGB, gV + (size_t)chunk(j) * G1 * RGB, bytes, mbs + MB_C + slot);
+            if (++slot == NR) { slot = 0; ++use; }
+          }
+        }
+        __syncwarp();
+      } else {
+        const int cg = (NB == 16) ? warp & 1 : 0;                    // this warp's columns
+        const int ush = (G1 == 8) ? 2 : 1, upc = 1 << ush;           // units of 16 rows per chunk
+        // at most NR chunks from one unit of a warp to its next: the parity
+        // of a slot's barrier then tells its uses apart
+        const int w0 = (NB == 16) ? (warp - 2) >> 1 : warp - 2, nw = min((NB == 16) ? 7 : 14, NR * upc);
+        const int c = cg * 8 + (lane & 7), drp = lane >> 3;
+        const bool live = c < nb;
+        const double* col = s_cp[c];
+        const int dec = (live && s_Ec[c] > -8000) ? s_Ec[c] + 1022 : 1 << 20;
+        // rows 16 p + 2 drp + {0, 1, 8, 9} of unit g (chunk g / upc, p = g %
+        // upc); rows past the last one read what follows in the scratch
+        // region and count as zero
+        double2 xa, xb;
+        int2 ea, eb;
+        auto load_u = [&](int g) {
+          const int r = chunk(j0 + (g >> ush)) * G1 * 8 + (g & (upc - 1)) * 16 + 2 * drp;
+          xa = __ldcg(reinterpret_cast<const double2*>(col + r));
+          xb = __ldcg(reinterpret_cast<const double2*>(col + r + 8));
+          ea = __ldcg(reinterpret_cast<const int2*>(ver + r));
+          eb = __ldcg(reinterpret_cast<const int2*>(ver + r + 8));
+        };
+        const int ug = w0 < nw ? (j1 - j0) * upc : 0;
+        if (w0 < ug) load_u(w0);
+        int s = slot0 + (w0 >> ush), u = use0;  // w0 >> ush < NR
+        if (s >= NR) { s -= NR; ++u; }
+        for (int g = w0; g < ug; g += nw) {
+          const int j = j0 + (g >> ush), p = g & (upc - 1);
+          const int r = chunk(j) * G1 * 8 + p * 16 + 2 * drp;
+          unsigned h1[4], h2[4];
+          bool ng[4];
+          const double xn[4] = {xa.x, xa.y, xb.x, xb.y};
+          const int en[4] = {ea.x, ea.y, eb.x, eb.y};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            // |x| 2^(Er - Ec) as a 64-bit fraction, then 56 bits rounded to
+            // nearest: digits 0-3 in h1, 4-7 in h2 at bits 29-23, 22-16, 15-9, 8-2
+            const unsigned long long b = (unsigned long long)__double_as_longlong(xn[q]);
+            const int e = (int)((b >> 52) & 0x7FFu);
+            const int sh = min(dec - en[q] - e, 63);
+            const bool z = e == 0 || r + (q & 1) + 8 * (q >> 1) >= Ld;
+            const unsigned long long m = (b << 11) | 0x8000000000000000ull;
+            const unsigned long long T = (m >> (z ? 63 : sh)) + 0x80ull;
+            h1[q] = (unsigned)(T >> 34);
+            h2[q] = (unsigned)(T >> 6);
+            ng[q] = (long long)b < 0;
+          }
+          if (g + nw < ug) load_u(g + nw);
+          if (j >= NR) mb_wait(MB_F + s, u - 1, ok);
+          unsigned char* pp = sC + s * CBB + (p * 2 * ND * NG + cg) * 128 + (lane & 7) * 16 + drp * 4;
+#pragma unroll
+          for (int q = 0; q < 4; q += 2) {
+            unsigned sg, nb2;
+            sign2(ng[q], ng[q + 1], sg, nb2);
+            const unsigned w[4] = {__byte_perm(h1[q], h1[q + 1], 0x7632), __byte_perm(h1[q], h1[q + 1], 0x5410),
+                                   __byte_perm(h2[q], h2[q + 1], 0x7632), __byte_perm(h2[q], h2[q + 1], 0x5410)};
+#pragma unroll
+            for (int l = 0; l < ND; ++l) {
+              const int bit = (l & 2) ? ((l & 1) ? 2 : 9) : ((l & 1) ? 0 : 7);
+              const unsigned d = ((w[l >> 1] >> bit) & 0x007F007Fu) | 0x43004300u;
+              *reinterpret_cast<unsigned*>(pp + (q >> 1) * ND * NG * 128 + l * NG * 128) = bf16x2_fma(d, sg, nb2);
+            }
+          }
+          fence_proxy_async();  // the digits before the MMAs read them
+          __syncwarp();
+          if (lane == 0) mbar_arrive(mbs + MB_C + s, 8 >> (ush + NG - 1));
+          s += ((g + nw) >> ush) - (g >> ush);  // at most NR on
+          if (s >= NR) { s -= NR; ++u; }
+        }
+      }
+      use = j1 / NR;
+      slot = j1 - use * NR;
+      mb_wait(MB_F + (slot ? slot - 1 : NR - 1), slot ? use : use - 1, ok);  // chunk j1 - 1
+      if (__syncthreads_or(!ok)) {
         expired();
         return 1;
       }
-      if (jc + 1 < nch1) {
-        stage_c(row1(jc + 1), b ^ 1);
-        stage_v(row1(jc + 1), R1, b ^ 1);
+      flush();
+      __syncthreads();
+    }
+    for (int s = 0; s < NR; ++s)
+      if (((nch - s + NR - 1) / NR) & 1) mpar ^= 0x420u << s;  // uses of slot s
+    // Guard, first on the chunks still in shared memory (the last NR): sums
+    // of |leading digit| products per (reflector, column), a warp's 16
+    // reflectors x 8 columns x 16 rows; any rows' sum is a lower bound.
+    // Capped, so that they are exact integers and their order does not
+    // matter.
+    const int gmt = warp % MT, gnt = (warp / MT) % NG, gks = warp / (MT * NG);
+    float gacc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int j = max(0, nch - NR); j < nch; ++j) {
+      if (gks < (groups(j) >> 1)) {
+        const int s = j % NR, i3 = lane >> 3;
+        unsigned a[4], bq[2];
+        ldsm_x4_t(a, sV + s * G1 * RGB + (2 * gks + (i3 >> 1)) * RGB + (2 * gmt + (i3 & 1)) * 128 + (lane & 7) * 16);
+        ldsm_x2(bq, sC + s * CBB + ((2 * gks + (i3 & 1)) * ND * NG + gnt) * 128 + (lane & 7) * 16);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] &= ABS2;
+        bq[0] &= ABS2;
+        bq[1] &= ABS2;
+        mma_bf16(gacc, a, bq);
       }
-      if (mw) {
-        const unsigned short* sAb = sV + b * BUF;
-        const unsigned short* sBb = sAb + BUF / 2;
-        const int r0 = sub * 16;
-        unsigned bq[ND][2];
+    }
+    __syncthreads();  // the slots are free
+    __shared__ int s_guard;
+    float* sG = reinterpret_cast<float*>(sV);  // KP x NB
+    // the FP64 rows, at the end of the work area until they are updated:
+    // V(r, t) (v0 on the diagonal, zero above) and C(r, c)
+    double* sTC = dyn + DYN_SMEM / 8 - r0d * NB;
+    double* sTV = sTC - r0d * kp;
+    for (int e = tid; e < KP * NB; e += NT) sG[e] = 0.f;
+    if (tid == 0) s_guard = 0;
+    for (int e = tid; e < r0d * kp; e += NT) {
+      const int r = e / kp, t = e - r * kp;
+      sTV[e] = (r > t) ? ldcg(I.V + (size_t)r * KM + t) : (r == t) ? cs.s_vt[t] : 0.0;
+    }
+    for (int e = tid; e < r0d * NB; e += NT) {
+      const int c = e / r0d, r = e - c * r0d;
+      sTC[r * NB + c] = ldcg(s_cp[c] - r0d + r);
+    }
+    __syncthreads();
+    if (gks < (G1 >> 1)) {
 #pragma unroll
-        for (int l = 0; l < ND; ++l) ldsm_x2(bq[l], sBb + (l * NBP + nt * 8 + (lane & 7)) * SB + r0 + ((lane >> 3) & 1) * 8);
-        const int ra = r0 + (lane & 7) + ((lane >> 4) << 3), qa = mt * 2 + ((lane >> 3) & 1);
+      for (int j = 0; j < 4; ++j) {
+        const int t = gmt * 16 + (lane >> 2) + ((j >> 1) << 3), c = gnt * 8 + 2 * (lane & 3) + (j & 1);
+        atomicAdd(sG + t * NB + c, fminf(gacc[j], 65536.f));
+      }
+    }
+    __syncthreads();
+    // the guard's test of (reflector t, column c): the digits' error (at
+    // most 2L 2^(es-57), 2^es the scale of D) must stay within
+    // gamma_L sum |v||c|, whose lower bound is 2^(es-14) sG + the FP64 rows'
+    // sum; a column without digit rows (all zero below r0d) has no digit
+    // error
+    auto guard_fails = [&](int t, int c) -> bool {
+      if (s_Ec[c] <= -8000 || sG[t * NB + c] >= GUARD1) return false;
+      double tabs = 0.0;
+      for (int r = t; r < r0d; ++r) tabs = fma(fabs(sTV[r * kp + t]), fabs(sTC[r * NB + c]), tabs);
+      const int es = s_Ec[c] + ebound(cs.s_vt[t]);
+      return !(ldexp((double)sG[t * NB + c], es - 14) + tabs >= ldexp((double)GUARD1, es - 14));
+    };
+    // D from the level sums (levels 0-4 and 5-8 exact in int64), the rows
+    // t .. r0d-1 in FP64 (V(r, t) = 0 above row t).  Lanes run over the
+    // columns here and below, so that a warp's rows end together (an FP64
+    // instruction costs a warp the same whatever its active lanes).
+    for (int o = tid; o < kp * NB; o += NT) {
+      const int c = o % NB, t = o / NB;
+      if (c >= nb) continue;
+      long long hi = 0, lo = 0;
 #pragma unroll
-        for (int k = 0; k < ND; ++k) {
-          unsigned a[4];
-          ldsm_x4_t(a, vaddr(sAb, R1, k, ra, qa));
+      for (int lam = 0; lam < 5; ++lam) hi = (hi << 7) + sF[(lam * KP + t) * NB + (c ^ (t & (NB - 1)))];
 #pragma unroll
-          for (int l = 0; l < ND && k + l < NLV; ++l) mma_bf16(acc[k + l], a, bq[l]);
-          if (k == 0) {
-            const unsigned ga[4] = {a[0] & ABS2, a[1] & ABS2, a[2] & ABS2, a[3] & ABS2};
-            const unsigned gb[2] = {bq[0][0] & ABS2, bq[0][1] & ABS2};
-            mma_bf16(gacc, ga, gb);
-          }
+      for (int lam = 5; lam < NLV; ++lam) lo = (lo << 7) + sF[(lam * KP + t) * NB + (c ^ (t & (NB - 1)))];
+      double tri0 = 0.0, tri1 = 0.0;
+      int r = t;
+#pragma unroll 4
+      for (; r + 1 < r0d; r += 2) {
+        tri0 = fma(sTV[r * kp + t], sTC[r * NB + c], tri0);
+        tri1 = fma(sTV[(r + 1) * kp + t], sTC[(r + 1) * NB + c], tri1);
+      }
+      if (r < r0d) tri0 = fma(sTV[r * kp + t], sTC[r * NB + c], tri0);
+      const int es = s_Ec[c] + ebound(cs.s_vt[t]);  // 2^Ft: the reflector's scale
+      const double dig = ll_scaled(hi, es - 42) + ll_scaled(lo, es - 70);
+      cs.s_D[t * CB + c] = dig + (tri0 + tri1);
+      // |sum| <= sum of |products|: |dig| >= 2^(es-3) needs no further test
+      if (ebound(dig) <= es - 3 && guard_fails(t, c)) s_guard |= 1;
+    }
+    __syncthreads();
+    if (s_guard && nch > 2) {
+      // the whole sums before the batch is handed over: 32 rows' leading
+      // digits at a time
+      float* fV = sG + KM * CB;   // 32 x KP
+      float* fC = fV + 32 * KP;   // 32 x NB
+      float ga[2] = {0.f, 0.f};
+      const unsigned short* vd = reinterpret_cast<const unsigned short*>(gV);
+      for (int rb = 0; rb < Ld; rb += 32) {
+        __syncthreads();
+        for (int e = tid; e < 32 * KP; e += NT) {
+          const int r = rb + e / KP, t = e % KP;
+          const unsigned short w = r < Ld ? __ldcg(vd + ((size_t)(r >> 3) * ND * (KP >> 3) + (t >> 3)) * 64 + (r & 7) * 8 + (t & 7)) : 0;
+          fV[e] = __uint_as_float((unsigned)(w & 0x7FFFu) << 16);
+        }
+        for (int e = tid; e < 32 * NB; e += NT) {
+          const int c = e >> 5, r = rb + (e & 31);
+          float d = 0.f;
+          if (c < nb && r < Ld && s_Ec[c] > -8000)
+            d = (float)(unsigned)(fix56(ldcg(s_cp[c] + r), ldcg(ver + r) + 56 - s_Ec[c]) >> 49);
+          fC[(e & 31) * NB + c] = d;
+        }
+        __syncthreads();
+        for (int k = 0; k < 2; ++k) {
+          const int o = tid + k * NT, c = o % NB, t = o / NB;
+          if (t < kp)
+            for (int r = 0; r < 32; ++r) ga[k] = fmaf(fV[r * KP + t], fC[r * NB + c], ga[k]);
         }
       }
-      if (jc + 1 < nch1) {
-        cp_wait_all();  // the next chunk's C values (its V digits may still be in flight)
-        __syncthreads();
-        digits_c(b ^ 1);
+      __syncthreads();
+      if (tid == 0) s_guard = 0;
+      for (int k = 0; k < 2; ++k) {
+        const int o = tid + k * NT;
+        if (o < kp * NB) sG[o] = ga[k];
       }
-      since += 16;
-      if (mw && (since == 128 || jc + 1 == nch1)) {
-#pragma unroll
-        for (int l = 0; l < NEX; ++l)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            atomicAdd(sF + ((cmb * NEX + l) * 32 + lane) * 4 + j, __float2int_rn(acc[l][j]));
-            acc[l][j] = 0.f;
-          }
+      __syncthreads();
+      for (int o = tid; o < kp * NB; o += NT) {
+        const int c = o % NB, t = o / NB;
+        if (c < nb && ebound(cs.s_D[t * CB + c]) <= s_Ec[c] + ebound(cs.s_vt[t]) - 3 && guard_fails(t, c)) s_guard = 1;
       }
-      if (since == 128) since = 0;
+      __syncthreads();
     }
-    // levels NEX .. 8 summed over the sub-blocks in order, then D from the
-    // level sums
-    __syncthreads();
-    constexpr int NST = NLV - NEX + 1;  // staged FP32 sums per warp: levels NEX .. 8 and the guard
-    float* sStage = reinterpret_cast<float*>(sV);                                 // MW x NST x 32 x 4
-    double* sL = reinterpret_cast<double*>(reinterpret_cast<char*>(sV) + 73728);  // NLV x 32 x NBP
-    __shared__ int s_guard;
-    if (tid == 0) s_guard = 0;
-    if (mw) {
-#pragma unroll
-      for (int l = NEX; l < NLV; ++l)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) sStage[((warp * NST + l - NEX) * 32 + lane) * 4 + j] = acc[l][j];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) sStage[((warp * NST + NST - 1) * 32 + lane) * 4 + j] = gacc[j];
-    }
-    __syncthreads();
-    // the guard's sums of |leading digit| products per (reflector, column),
-    // added over the four row sub-blocks (checked with D below)
-    float* sG = reinterpret_cast<float*>(reinterpret_cast<char*>(sV) + 32768);  // KM x CB
-    for (int e = tid; e < COMBOS * 128; e += NT) {
-      const int j = e & 3, ln = (e >> 2) & 31, cb = e >> 7;
-      const int t = (cb % KT) * 16 + (ln >> 2) + ((j >> 1) << 3), c = (cb / KT) * 8 + 2 * (ln & 3) + (j & 1);
-      if (t < kp && c < nb) {
-        float g = 0.f;
-        for (int sb = 0; sb < 4; ++sb) g += sStage[(((sb * COMBOS + cb) * NST + NST - 1) * 32 + ln) * 4 + j];
-        sG[t * CB + c] = g;
-      }
-    }
-    for (int e = tid; e < COMBOS * NLV * 128; e += NT) {
-      const int j = e & 3, ln = (e >> 2) & 31, lam = (e >> 7) % NLV, cb = (e >> 7) / NLV;
-      double v = 0.0;
-      if (lam < NEX) {
-        v = (double)sF[((cb * NEX + lam) * 32 + ln) * 4 + j];
-      } else {
-        for (int sb = 0; sb < 4; ++sb)
-          v += (double)sStage[(((sb * COMBOS + cb) * NST + lam - NEX) * 32 + ln) * 4 + j];
-      }
-      const int t = (cb % KT) * 16 + (ln >> 2) + ((j >> 1) << 3), c = (cb / KT) * 8 + 2 * (ln & 3) + (j & 1);
-      sL[(lam * 32 + t) * NBP + c] = v;
-    }
-    __syncthreads();
-    for (int o = tid; o < kp * nb; o += NT) {
-      const int t = o / nb, c = o - t * nb;
-      double s = sL[((NLV - 1) * 32 + t) * NBP + c];
-      for (int lam = NLV - 2; lam >= 0; --lam) s = fma(s, 0x1p-7, sL[(lam * 32 + t) * NBP + c]);
-      // rows t .. r0d-1 in FP64 (V(r, t) = 0 above row t), with sum |v||c|
-      const double* col = commit_col(cs.s_cid, c);
-      double tri = 0.0, tabs = 0.0;
-      for (int r = t; r < r0d; ++r) {
-        const double vr = (r > t) ? ldcg(I.V + (size_t)r * KM + t) : cs.s_vt[t], cr = ldcg(col + r);
-        tri = fma(vr, cr, tri);
-        tabs = fma(fabs(vr), fabs(cr), tabs);
-      }
-      const int es = s_Ec[c] + ebound(cs.s_vt[t]);  // 2^Ft: the reflector's scale
-      cs.s_D[t * CB + c] = ldexp(s, es - 14) + tri;
-      // guard: the digits' error (at most 2L 2^(es-57)) must stay within
-      // gamma_L sum |v||c|, whose lower bound is 2^(es-14) sG + tabs; a
-      // column without digit rows (all zero below r0d) has no digit error
-      if (s_Ec[c] > -8000 && !(ldexp((double)sG[t * CB + c], es - 14) + tabs >= ldexp((double)GUARD1, es - 14)))
-        s_guard = 1;
-    }
-    __syncthreads();
-    // bf16 MMAs of pass 1: per chunk, each MMA warp's 16 rows take the 43
-    // digit pairs and the guard's
-    const double mma1 = (double)MW * nch1 * 44.0;
+    // MMA work in units of m16n8k16: pass 1, then pass 2 below
+    double mma1 = 0.0;
+    for (int mt = 0; mt < MT; ++mt) mma1 += 8.0 * NG * tile_digits<NB>(mt, MT) * (0.5 * ngr);
     if (s_guard || I.guard_force == 1) {
       if (tid == 0) {
         atomicAdd(I.ctl + C_GUARD1, 1);
@@ -2198,138 +2445,222 @@ struct Engine {
       return 2;
     }
     // D' = T^T D
-    for (int o = tid; o < kp * nb; o += NT) {
-      const int t = o % kp, cc = o / kp;
-      double e2 = 0.0;
-      for (int sidx = 0; sidx <= t; ++sidx) e2 = fma(cs.s_T[t * (t + 1) / 2 + sidx], cs.s_D[sidx * CB + cc], e2);
-      cs.s_E[t * CB + cc] = e2;
+    for (int o = tid; o < kp * NB; o += NT) {
+      const int c = o % NB, t = o / NB;
+      double e0 = 0.0, e1 = 0.0;
+      const double* tr = cs.s_T + t * (t + 1) / 2;
+      int q = 0;
+      for (; q + 1 <= t; q += 2) {
+        e0 = fma(tr[q], cs.s_D[q * CB + c], e0);
+        e1 = fma(tr[q + 1], cs.s_D[(q + 1) * CB + c], e1);
+      }
+      if (q <= t) e0 = fma(tr[q], cs.s_D[q * CB + c], e0);
+      cs.s_E[t * CB + c] = (c < nb) ? e0 + e1 : 0.0;
     }
     __syncthreads();
-    // digits of D' under a column scale: warp c, lane t
-    for (int c = warp; c < NBP; c += NW) {
-      const double v = (c < nb && lane < kp) ? scale2(cs.s_E[lane * CB + c], ebound(cs.s_vt[lane])) : 0.0;
-      const int ee = __reduce_max_sync(0xffffffffu, ebound(v));
-      unsigned ha, la;
-      halves28(fix56(v, 56 - ee), ha, la);
-      const unsigned hb = __shfl_down_sync(0xffffffffu, ha, 1), lb = __shfl_down_sync(0xffffffffu, la, 1);
-      const bool nega = v < 0.0;
-      const bool negb = __shfl_down_sync(0xffffffffu, nega ? 1 : 0, 1) != 0;
-      unsigned sg, nb2;
-      sign2(nega, negb, sg, nb2);
-      if ((lane & 1) == 0) {
-#pragma unroll
-        for (int k = 0; k < ND; ++k) *reinterpret_cast<unsigned*>(sE + (k * NBP + c) * SE + lane) = dig2k(k, ha, la, hb, lb, sg, nb2);
+    // the FP64 rows; rows kp .. r0d-1 belong to the trailing norm and are
+    // kept (in D's place) for the sum per column below
+    double* s_tx = cs.s_D;
+    for (int o = tid; o < r0d * NB; o += NT) {
+      const int c = o % NB, r = o / NB;
+      if (c >= nb) continue;
+      double x = sTC[r * NB + c], x1 = 0.0;
+      const int te = min(r + 1, kp);
+      int t = 0;
+      for (; t + 1 < te; t += 2) {
+        x = fma(-sTV[r * kp + t], cs.s_E[t * CB + c], x);
+        x1 = fma(-sTV[r * kp + t + 1], cs.s_E[(t + 1) * CB + c], x1);
       }
+      if (t < te) x = fma(-sTV[r * kp + t], cs.s_E[t * CB + c], x);
+      x += x1;
+      s_cp[c][r - r0d] = x;
+      if (r >= kp) s_tx[(r - kp) * NB + c] = x;
+    }
+    // ---- pass 2: V tiles of 128 rows, two buffers (one for KP > 32)
+    unsigned char* sE = base + 2 * KM * CB * 8;        // digits of D''
+    unsigned char* sW = sE + KP / 8 * NPL * NG * 128;
+    const bool dbl = KP <= 32;
+    const int nt2 = (ngr + 15) / 16;
+    const int s2 = tm.rank % nt2;
+    auto tile = [&](int i) { const int t = i + s2; return t >= nt2 ? t - nt2 : t; };
+    auto stage_t = [&](int i) {  // one thread
+      const int b = dbl ? i & 1 : 0;
+      const unsigned bytes = (unsigned)min(16, ngr - tile(i) * 16) * RGB;
+      mbar_expect_tx(mbs + MB_V + b, bytes);
+      bulk_g2s(sW + b * 16 * RGB, gV + (size_t)tile(i) * 16 * RGB, bytes, mbs + MB_V + b);
+    };
+    fence_proxy_async();  // the work area's generic accesses before the async copies
+    __syncthreads();
+    if (tid == 0) {
+      stage_t(0);
+      if (dbl && nt2 > 1) stage_t(1);
+    }
+    // digits of D'' = 2^Ft D' under a column scale (a warp per column, lane t
+    // holds reflectors t and t + 32): [reflector group][digit][column group]
+    // blocks
+    for (int c = warp; c < NB; c += NW) {
+      double v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int t = lane + 32 * h;
+        v[h] = (t < kp) ? scale2(cs.s_E[t * CB + c], ebound(cs.s_vt[t])) : 0.0;
+      }
+      const int ee = __reduce_max_sync(0xffffffffu, max(ebound(v[0]), ebound(v[1])));
       if (lane == 0) s_Ee[c] = ee;
-    }
-    __syncthreads();
-    // ---- pass 2 (digit rows r0d .. L-1; rows below r0d after the loop)
-    const int nch2 = (Ld + R2 - 1) / R2;
-    const bool act2 = warp < 8 * NTN;
-    const int rt = warp & 7, nt2 = warp >> 3;
-    const int c0 = nt2 * 8 + 2 * tq;
-    double nrm0 = 0.0, nrm1 = 0.0;
-    const int s2 = tm.rank % nch2;
-    auto row2 = [&](int jc) { return ((jc + s2) % nch2) * R2; };
-    fence_proxy_async();  // pass-1 scratch writes before the async copies
-    __syncthreads();
-    stage_v(row2(0), R2, 0);
-    for (int jc = 0; jc < nch2; ++jc) {
-      const int rb = row2(jc), b = jc & 1;
-      const bool okv = wait_v(b);
-      if (__syncthreads_or(!okv)) {
-        expired();
-        return 1;
-      }
-      if (jc + 1 < nch2) stage_v(row2(jc + 1), R2, b ^ 1);
-      if (act2) {
-        // this thread's four elements: rows ra, ra + 8; columns c0, c0 + 1
-        const int ra = r0d + rb + rt * 16 + g, rb8 = ra + 8;
-        double xv[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = c0 + (j & 1), row = (j < 2) ? ra : rb8;
-          xv[j] = (act2 && c < nb && row < L) ? ldcg(commit_col(cs.s_cid, c) + row) : 0.0;
-        }
-        const int er0 = (ra < L) ? ldcg(I.Ver + ra) : 0, er1 = (rb8 < L) ? ldcg(I.Ver + rb8) : 0;
-        float a2[NLV][4];
+      for (int h = 0; h < 2; ++h) {
+        if (32 * h >= KP) break;
+        unsigned ha, la;
+        halves28(fix56(v[h], 56 - ee), ha, la);
+        const unsigned hb = __shfl_down_sync(0xffffffffu, ha, 1), lb = __shfl_down_sync(0xffffffffu, la, 1);
+        const bool nega = v[h] < 0.0;
+        const bool negb = __shfl_down_sync(0xffffffffu, nega ? 1 : 0, 1) != 0;
+        unsigned sg, nb2;
+        sign2(nega, negb, sg, nb2);
+        const int t = lane + 32 * h;
+        if ((lane & 1) == 0 && t < KP) {
+          unsigned char* p = sE + ((t >> 3) * NPL * NG + (c >> 3)) * 128 + (c & 7) * 16 + (t & 7) * 2;
 #pragma unroll
-        for (int l = 0; l < NLV; ++l)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) a2[l][j] = 0.f;
-        const unsigned short* sAb = sV + b * BUF;
-        const int r0 = rt * 16, rq = r0 + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-        for (int ks = 0; ks < KT; ++ks) {
-          unsigned eb[ND][2];
-#pragma unroll
-          for (int l = 0; l < ND; ++l)
-            ldsm_x2(eb[l], sE + (l * NBP + nt2 * 8 + (lane & 7)) * SE + ks * 16 + ((lane >> 3) & 1) * 8);
-#pragma unroll
-          for (int k = 0; k < ND; ++k) {
-            unsigned a[4];
-            ldsm_x4(a, vaddr(sAb, R2, k, rq, ks * 2 + ((lane >> 4) & 1)));
-#pragma unroll
-            for (int l = 0; l < ND && k + l < NLV; ++l) mma_bf16(a2[k + l], a, eb[l]);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int row = (j < 2) ? ra : rb8;
-          const int c = c0 + (j & 1);
-          if (c < nb && row < L) {
-            double* p = commit_col(cs.s_cid, c);
-            long long u = 0;
-#pragma unroll
-            for (int l = 0; l < 7; ++l) u += (long long)__float2int_rn(a2[l][j]) * (1ll << (43 - 7 * l));
-            u += (long long)(__float2int_rn(a2[7][j]) >> 6);
-            u += (long long)(__float2int_rn(a2[8][j]) >> 13);
-            const int es = max(-2044, ((j < 2) ? er0 : er1) + s_Ee[c] - 57);
-            const double x = xv[j] - ll_scaled(u, es);
-            p[row] = x;
-            if (row >= kp) {
-              if (j & 1) nrm1 = fma(x, x, nrm1);
-              else nrm0 = fma(x, x, nrm0);
-            }
-          }
+          for (int l = 0; l < NPL; ++l)
+            *reinterpret_cast<unsigned*>(p + l * NG * 128) = l < ND ? dig2k(l, ha, la, hb, lb, sg, nb2) : 0u;
         }
       }
     }
-    // rows r < r0d in FP64, in the order of the FP64 commit; rows kp .. r0d-1
-    // belong to the trailing norm: kept for a fixed-order sum per column (in
-    // rows 8 .. 15 of s_nrm, which the row tiles below leave free)
-    double* s_tx = cs.s_nrm + 8 * CB;
-    for (int o = tid; o < r0d * nb; o += NT) {
-      const int r = o / nb, c = o - r * nb;
-      double* col = commit_col(cs.s_cid, c);
-      double x = ldcg(col + r);
-      for (int t = 0; t <= min(r, kp - 1); ++t)
-        x = fma(-((r > t) ? ldcg(I.V + (size_t)r * KM + t) : cs.s_vt[t]), cs.s_E[t * CB + c], x);
-      col[r] = x;
-      if (r >= kp) s_tx[(r - kp) * CB + c] = x;
-    }
-    // trailing norms: lanes of one column quad, then the 8 row tiles in order
+    // A warp reads its own lane quadrant; the four warps of a quadrant share
+    // the column pairs.
+    constexpr int PQ = NG;  // column pairs per warp
+    const int rl = 32 * (warp & 3) + lane, pw = warp >> 2;
+    double nrm[PQ][2];
 #pragma unroll
-    for (int o = 4; o < 32; o <<= 1) {
-      nrm0 += __shfl_xor_sync(0xffffffffu, nrm0, o);
-      nrm1 += __shfl_xor_sync(0xffffffffu, nrm1, o);
+    for (int q = 0; q < PQ; ++q) nrm[q][0] = nrm[q][1] = 0.0;
+    // MMAs of tile i into accumulator half i & 1: by warp i mod NW, so that the
+    // time an issuing warp loses (about 1000 cycles) spreads over all of them
+    auto issue2 = [&](int i) {
+      if (mma_thread(i & (NW - 1))) {
+        mb_wait(MB_V + (dbl ? i & 1 : 0), dbl ? i >> 1 : i, ok);
+        if (i >= 2) mb_wait(MB_T + (i & 1), (i >> 1) - 1, ok);
+        if (ok) {
+          tc_fence_after();
+          const unsigned av = smem_u32(sW + (dbl ? i & 1 : 0) * 16 * RGB), bv = smem_u32(sE);
+          const unsigned acc0 = tmem + (i & 1) * 256;
+          switch (MT) {
+            case 1: issue_pass2<NB, 1>(av, bv, acc0); break;
+            case 2: issue_pass2<NB, 2>(av, bv, acc0); break;
+            case 3: issue_pass2<NB, 3>(av, bv, acc0); break;
+            default: issue_pass2<NB, 4>(av, bv, acc0); break;
+          }
+          umma_commit(mbs + MB_F + (i & 1));
+        }
+      }
+      __syncwarp();
+    };
+    fence_proxy_async();  // the digits before the MMAs read them
+    __syncthreads();
+    // level sums -> u -> x -= u 2^(Er+Ee-57), norms; a pair's columns are
+    // loaded before the pair ahead of it is worked on
+    double xn[2];
+    int en = 0;
+    auto load_x = [&](int i, int pr) {
+      const int r = min(tile(i) * 128 + rl, Ld - 1);
+      en = ldcg(ver + r);
+      xn[0] = ldcg(s_cp[2 * pr] + r);
+      xn[1] = ldcg(s_cp[2 * pr + 1] + r);
+    };
+    load_x(0, pw);
+    issue2(0);
+    for (int i = 0; i < nt2; ++i) {
+      if (dbl && i + 1 < nt2) issue2(i + 1);
+      mb_wait(MB_F + (i & 1), i >> 1, ok);
+      if (tid == 32 * (i & (NW - 1)) && ok) {  // tile i's V buffer is free
+        const int nx = i + (dbl ? 2 : 1);
+        if (nx < nt2) stage_t(nx);
+      }
+      __syncwarp();
+      tc_fence_after();
+      const int r = tile(i) * 128 + rl;
+#pragma unroll
+      for (int q = 0; q < PQ; ++q) {
+        const int pr = pw + 4 * q;
+        float lv[NLV][2];
+        const unsigned a0 = tmem + ((unsigned)(32 * (warp & 3)) << 16) + (i & 1) * 256 + 2 * pr;
+#pragma unroll
+        for (int l = 0; l < NLV; ++l) tmem_ld<2>(lv[l], a0 + l * NB);
+        const double x2[2] = {xn[0], xn[1]};
+        const int er = en;
+        if (q + 1 < PQ) load_x(i, pr + 4);
+        else if (i + 1 < nt2) load_x(i + 1, pw);
+        tmem_ld_wait();
+        if (q + 1 == PQ) {  // this warp's accumulators are read
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(mbs + MB_T + (i & 1), 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          int lq[NLV];
+#pragma unroll
+          for (int l = 0; l < NLV; ++l) {
+            // |level| < 2^22 for l <= 3, and for every l with KP <= 32: the
+            // integer is the low mantissa of level + 1.5 2^23
+            if (l <= 3 || KP <= 32) lq[l] = __float_as_int(lv[l][u] + 12582912.f) - 0x4B400000;
+            else lq[l] = __float2int_rn(lv[l][u]);
+          }
+          const long long uu = ((long long)(lq[0] * 128 + lq[1]) << 36) + ((long long)(lq[2] * 128 + lq[3]) << 22) +
+                               ((long long)(lq[4] * 128 + lq[5]) << 8) +
+                               (long long)(lq[6] * 2 + (lq[7] >> 6) + (lq[8] >> 13));
+          const int c = 2 * pr + u;
+          if (r < Ld && c < nb) {
+            const int es = max(-2044, er + s_Ee[c] - 57);
+            const double xv = x2[u] - ll_scaled(uu, es);
+            s_cp[c][r] = xv;
+            nrm[q][u] = fma(xv, xv, nrm[q][u]);
+          }
+        }
+      }
+      if (!dbl && i + 1 < nt2) issue2(i + 1);
     }
-    if (act2 && lane < 4) {
-      cs.s_nrm[rt * CB + nt2 * 8 + 2 * lane] = nrm0;
-      cs.s_nrm[rt * CB + nt2 * 8 + 2 * lane + 1] = nrm1;
+    {
+      const int n0 = (nt2 + 1) >> 1, n1 = nt2 >> 1;  // uses of the two halves
+      if (n0 & 1) mpar ^= (1u << MB_F) | (1u << MB_T);
+      if (n1 & 1) mpar ^= (2u << MB_F) | (2u << MB_T);
+      if ((dbl ? n0 : nt2) & 1) mpar ^= 1u << MB_V;
+      if (dbl && (n1 & 1)) mpar ^= 2u << MB_V;
+    }
+    if (__syncthreads_or(!ok)) {
+      expired();
+      return 1;
+    }
+    // trailing norms: 8 partials of 16 rows per column, then in order with
+    // the kept rows
+    double* sN = reinterpret_cast<double*>(sE);  // NB x 129
+    double* sP = sN + 129 * NB;                  // 8 x NB
+#pragma unroll
+    for (int q = 0; q < PQ; ++q) {
+      sN[2 * (pw + 4 * q) * 129 + rl] = nrm[q][0];
+      sN[(2 * (pw + 4 * q) + 1) * 129 + rl] = nrm[q][1];
+    }
+    __syncthreads();
+    if (tid < 8 * NB) {
+      const int c = tid % NB, p = tid / NB;
+      double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 16; k += 2) {
+        v0 += sN[c * 129 + p * 16 + k];
+        v1 += sN[c * 129 + p * 16 + k + 1];
+      }
+      sP[p * NB + c] = v0 + v1;
     }
     __syncthreads();
     if (tid < nb) {
       double v = 0.0;
-      for (int r8 = 0; r8 < 8; ++r8) v += cs.s_nrm[r8 * CB + tid];
-      for (int r = kp; r < r0d; ++r) v = fma(s_tx[(r - kp) * CB + tid], s_tx[(r - kp) * CB + tid], v);
+      for (int p = 0; p < 8; ++p) v += sP[p * NB + tid];
+      for (int r = kp; r < r0d; ++r) v = fma(s_tx[(r - kp) * NB + tid], s_tx[(r - kp) * NB + tid], v);
       if (cs.s_cid[tid] >= 0) I.u[cs.s_cid[tid]] = sqrt(v);
     }
-    if (tid == 0 && I.phase_ns)  // pass 2: 43 digit pairs per 16 x 8 tile and 16 reflectors
-      atomicAdd(I.phase_ns + 2 * NPHASE, mma1 + (double)(8 * NTN) * nch2 * KT * 43.0);
+    if (tid == 0 && I.phase_ns)  // pass 2: 43 digit pairs per tile and 16 reflectors
+      atomicAdd(I.phase_ns + 2 * NPHASE, mma1 + 8.0 * NG * 43.0 * MT * nt2);
     return 0;
   }
-
 
   // Commit for kp <= 4 (one-column LH steps and short J): V staged once for
   // all L rows, then one warp per column does D = V^T x (lanes over rows,
@@ -2451,16 +2782,12 @@ struct Engine {
       nP += kp;
       return sync();
     }
-    const int VS = kp | 1;                          // odd row stride of staged V rows
     double* s_D = dyn;                              // KM x CB
     double* s_E = dyn + KM * CB;                    // KM x CB
     double* wk = dyn + 2 * KM * CB;                 // work area
     constexpr int WKD = DYN_SMEM / 8 - 2 * KM * CB; // its size in doubles
-    const int RC1 = min(1024, (WKD / (VS + CB)) & ~31);  // pass-1 rows per chunk
-    const int RC2 = (WKD / VS >= 512) ? 512 : (WKD / VS >= 256) ? 256 : (WKD / VS >= 128) ? 128 : 64;
     __shared__ double s_T[KM * KM / 2 + KM];
     __shared__ double s_vt[KM];
-    __shared__ double s_nrm[NW * CB];
     __shared__ int s_cid[CB];
     __shared__ int s_list[CAND_LOCAL_MAX + 1];
     for (int e = tid; e < kp * kp; e += NT) {
@@ -2481,39 +2808,34 @@ struct Engine {
       nP += kp;
       return sync();
     }
-    const CommitShape cs{L, RC1, RC2, VS, wk, s_D, s_E, s_T, s_vt, s_nrm, s_cid};
-    // the tensor-core form needs this panel's reflector digits
-    const bool tc = vd_ok && kp > 4 && kp <= 32 && L <= 16384 && L >= kp + 72;  // int32 level sums
-    for (int base = 0; base < nl; base += CB) {
-      const int nb = min(CB, nl - base);
-      __syncthreads();
-      if (tid < nb) s_cid[tid] = s_list[base + tid];
-      __syncthreads();
-      if (tc) {
-        int r;
-        if (kp <= 16) r = (nb <= 8) ? commit_tc<8, 1>(cs, nb) : commit_tc<16, 1>(cs, nb);
-        else r = (nb <= 8) ? commit_tc<8, 2>(cs, nb) : commit_tc<16, 2>(cs, nb);
-        if (r == 1) return false;
-        if (r == 0) continue;
-        __syncthreads();  // r == 2: the FP64 commit below takes this batch
-      }
-      switch (nb) {
-        case 1: commit_batch<1>(cs); break;
-        case 2: commit_batch<2>(cs); break;
-        case 3: commit_batch<3>(cs); break;
-        case 4: commit_batch<4>(cs); break;
-        case 5: commit_batch<5>(cs); break;
-        case 6: commit_batch<6>(cs); break;
-        case 7: commit_batch<7>(cs); break;
-        case 8: commit_batch<8>(cs); break;
-        case 9: commit_batch<9>(cs); break;
-        case 10: commit_batch<10>(cs); break;
-        case 11: commit_batch<11>(cs); break;
-        case 12: commit_batch<12>(cs); break;
-        case 13: commit_batch<13>(cs); break;
-        case 14: commit_batch<14>(cs); break;
-        case 15: commit_batch<15>(cs); break;
-        default: commit_batch<16>(cs); break;
+    const CommitShape cs{L, s_D, s_E, s_T, s_vt, s_cid};
+    // The tensor-core form needs this panel's reflector digits and int32 level
+    // sums.  It costs about 30 000 cycles per 16 columns and 30 L (8 columns
+    // or fewer) or 60 L beside them, the FP64 forms kp L per column: they are
+    // the shorter ones for few reflectors, rows or columns.
+    const bool can = vd_ok && kp > 4 && L <= 16384 && L >= kp + 72;
+    const bool fits = (size_t)L * ((kp | 1) + nl) + 2 * KM * 8 + 32 <= DYN_SMEM / 8;
+    const int nb16 = (nl + CB - 1) / CB, nb32 = (nl + 31) / 32;
+    const float tc_cost = nl <= 8 ? 30000.f + 30.f * L : nb16 * (30000.f + 60.f * L);
+    const bool test = I.guard_force != 0;  // the guard's test: the tensor-core form wherever it can run
+    const bool narrow = nl <= 8 && fits && (!can || (!test && (float)kp * L * nl + 8000.f < tc_cost));
+    const bool tc = can && !narrow && (test || nl <= 8 || tc_cost < nb32 * ((float)kp * L * 32.f + 6000.f));
+    if (narrow) {
+      commit_narrow(s_T, s_vt, s_list, nl, L);
+    } else if (!tc) {
+      commit_cols(s_T, s_vt, s_list, nl, L);
+    } else {
+      for (int base = 0; base < nl; base += CB) {
+        const int nb = min(CB, nl - base);
+        __syncthreads();
+        if (tid < nb) s_cid[tid] = s_list[base + tid];
+        __syncthreads();
+        const int r = (nb <= 8) ? commit_tc<8>(cs, nb) : commit_tc<16>(cs, nb);
+        if (r == 1) {
+          tc_failed = true;
+          return false;
+        }
+        if (r == 2) commit_cols(s_T, s_vt, s_list + base, nb, L);  // handed over by the accuracy guard
       }
     }
     nP += kp;
