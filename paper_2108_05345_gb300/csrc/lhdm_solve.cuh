@@ -56,7 +56,7 @@ struct Engine {
   // per-phase device time and algorithmic FP64 flops (rank 0, thread 0),
   // in shared memory so that no per-thread array forces the engine's state
   // into local memory
-  double* phf;
+  long long* phf;
 
   __device__ Engine(Team& t, const Inst& inst, double* d) : tm(t), I(inst), dyn(d) {
     tid = threadIdx.x;
@@ -64,21 +64,23 @@ struct Engine {
     warp = tid >> 5;
     sgn = I.prm.mode;
     nx = sgn ? 2 * I.n : I.n;
-    __shared__ double s_phf[2 * NPHASE];
+    __shared__ long long s_phf[2 * NPHASE];
     phf = s_phf;
     if (tid == 0)
-      for (int i = 0; i < 2 * NPHASE; ++i) s_phf[i] = 0.0;
+      for (int i = 0; i < 2 * NPHASE; ++i) s_phf[i] = 0;
   }
 
   // Counts algorithmic flops (an FMA is 2) of a phase; uniform state only.
-  __device__ __forceinline__ void flops(int p, double f) {
+  // In integers: the sums stand on rank 0's chain, and an FP64 instruction
+  // is 64 cycles of it.
+  __device__ __forceinline__ void flops(int p, long long f) {
     if (I.phase_ns && tm.rank == 0 && tid == 0) phf[NPHASE + p] += f;
   }
 
   __device__ __forceinline__ void phase(int p) {
     if (I.phase_ns && tm.rank == 0 && tid == 0) {
       const long long t = gtimer();
-      if (cur_phase >= 0) phf[cur_phase] += (double)(t - t_last);
+      if (cur_phase >= 0) phf[cur_phase] += t - t_last;
       t_last = t;
       cur_phase = p;
     }
@@ -100,6 +102,18 @@ struct Engine {
   __device__ __forceinline__ int phys(int e) const { return e >= I.n ? e - I.n : e; }
   __device__ __forceinline__ double pos_sign(int p) const {
     return sgn ? (double)ldcg(I.csign + ldcg(I.order + p)) : 1.0;
+  }
+
+  // *p where ok, else 0, without a branch (the other lanes read a word that
+  // is always there): a branch around each load kept the loads of a loop one
+  // after another, about 470 cycles each.
+  __device__ __forceinline__ double ldif(bool ok, const double* p) const {
+    const double v = ldcg(ok ? p : I.rhs);
+    return ok ? v : 0.0;
+  }
+  __device__ __forceinline__ int ldif(bool ok, const int* p) const {
+    const int v = ldcg(ok ? p : I.ctl);
+    return ok ? v : 0;
   }
 
   __device__ __forceinline__ double* Rcol(int slot) const { return I.R + (size_t)slot * I.ldr; }
@@ -242,7 +256,8 @@ struct Engine {
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int t = t0 + lane + 32 * j;
-        v[j] = (t < tm.size) ? ldcg(I.part + (size_t)t * PW + P_O1 + f) : (is_max ? -INFINITY : 0.0);
+        const double x = ldcg(I.part + (size_t)min(t, tm.size - 1) * PW + P_O1 + f);
+        v[j] = (t < tm.size) ? x : (is_max ? -INFINITY : 0.0);
       }
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc = is_max ? fmax(acc, v[j]) : acc + v[j];
@@ -260,8 +275,10 @@ struct Engine {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int t = t0 + lane + 32 * j;
-          v[j] = (t < tm.size) ? ldcg(I.part + (size_t)t * PW + P_O1) : 0.0;
-          ix[j] = (t < tm.size) ? ldcg(I.part + (size_t)t * PW + P_O1 + 1) : -1.0;
+          const double* p = I.part + (size_t)min(t, tm.size - 1) * PW + P_O1;
+          v[j] = ldcg(p);
+          ix[j] = ldcg(p + 1);
+          if (t >= tm.size) ix[j] = -1.0;
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) best = amax_merge(best, ArgMax{v[j], (int)ix[j]});
@@ -446,7 +463,7 @@ struct Engine {
     // (c) partial Gram matrix of the projected candidates over this CTA's rows
     const int L = I.m - nP;
     const int npair = KK * (KK + 1) / 2;
-    flops(PH_DM, 2.0 * npair * (double)L);
+    flops(PH_DM, 2ll * npair * L);
     {
       int q0, q1;
       split(L, tm.size, tm.rank, q0, q1);
@@ -578,7 +595,7 @@ struct Engine {
         double s = 0.0;
         for (int rr = max(q0, i + 1) + lane; rr < q1; rr += 32) {
           const double vi = ldcg(V + (size_t)rr * KM + i);
-          const double y = (l < k0) ? ldcg(V + (size_t)rr * KM + l) : ldcg(btp + rr);
+          const double y = ldcg(l < k0 ? V + (size_t)rr * KM + l : btp + rr);
           s = fma(y, vi, s);
         }
         s = warp_sum(s);
@@ -643,7 +660,7 @@ struct Engine {
           I.T[tid + i * KM] = -beta * ((a0 + a1) + (a2 + a3));
         }
       }
-      flops(PH_PANEL, 2.0 * (double)(2 * (k0 - i) + 1) * (double)(L - i));
+      flops(PH_PANEL, 2ll * (2 * (k0 - i) + 1) * (L - i));
       // update own rows r > i of the later columns and of b
       const int nl = k0 - i;  // columns i+1..k0-1 and b
       for (int e = tid; e < (q1 - max(q0, i + 1)) * nl; e += NT) {
@@ -763,7 +780,7 @@ struct Engine {
     __shared__ int s_stop, s_stop2;
     for (int e = tid; e < nr * NL; e += NT) {
       const int rr = e / NL, l = e - rr * NL;
-      sP[rr * PS + l] = (l < k0) ? ldcg(Wcol(s_J[l]) + nP + q0 + rr) : ldcg(I.bt + nP + q0 + rr);
+      sP[rr * PS + l] = ldcg((l < k0 ? Wcol(s_J[l]) : I.bt) + nP + q0 + rr);
     }
     if (tid < k0) s_an[tid] = ldcg(I.anorm + s_J[tid]);
     // Exponent bounds of the panel columns' norms: u_j for a selected
@@ -960,8 +977,8 @@ struct Engine {
           }
         }
       }
-      flops(PH_PANEL, 2.0 * (double)(2 * (k0 - i) + 1) * (double)(L - i));
-      if (two) flops(PH_PANEL, 2.0 * (double)(2 * (k0 - i - 1) + 1) * (double)(L - i - 1));
+      flops(PH_PANEL, 2ll * (2 * (k0 - i) + 1) * (L - i));
+      if (two) flops(PH_PANEL, 2ll * (2 * (k0 - i - 1) + 1) * (L - i - 1));
       // own rows: reflector i on rows > i (columns > i), then reflector i+1
       // on rows > i+1 (columns > i+1), both in two FMAs per element from
       // the row's columns i and i+1 before either reflector (columns i+2 ..
@@ -1068,7 +1085,7 @@ struct Engine {
           s_bt[i] = beta;
         }
       }
-      flops(PH_PANEL, 2.0 * (double)(2 * (k0 - i) + 1) * (double)(L - i));
+      flops(PH_PANEL, 2ll * (2 * (k0 - i) + 1) * (L - i));
       // update own rows > i of the later columns and of Q^T b
       const int nl = k0 - i;
       for (int e = tid; e < (nr - r0) * nl; e += NT) {
@@ -1123,54 +1140,78 @@ struct Engine {
     return true;
   }
 
-  // Back substitution with the kk x kk triangle R22 (one warp).
-  __device__ void solve_r22(int k, double* y) {
-    double a0 = (lane < k) ? ldcg(I.pr + lane) : 0.0;
-    double a1 = (lane + 32 < k) ? ldcg(I.pr + lane + 32) : 0.0;
-    // reciprocal diagonal computed by all lanes at once, off the chain
-    const double r0 = (lane < k) ? rcp_nr(ldcg(I.R22 + lane + lane * KM)) : 0.0;
-    const double r1 = (lane + 32 < k) ? rcp_nr(ldcg(I.R22 + (lane + 32) + (lane + 32) * KM)) : 0.0;
-    double y0 = 0.0, y1 = 0.0;
-    for (int jj = k - 1; jj >= 0; --jj) {
-      const int owner = jj & 31;
-      const bool hi = jj >= 32;
-      double yv = 0.0;
-      if (lane == owner) yv = (hi ? a1 : a0) * (hi ? r1 : r0);
-      yv = __shfl_sync(0xffffffffu, yv, owner);
-      if (lane == owner) { if (hi) y1 = yv; else y0 = yv; }
-      if (lane < jj) a0 -= ldcg(I.R22 + lane + jj * KM) * yv;
-      if (lane + 32 < jj) a1 -= ldcg(I.R22 + lane + 32 + jj * KM) * yv;
-    }
-    if (lane < k) y[lane] = y0;
-    if (lane + 32 < k) y[lane + 32] = y1;
-  }
-
   // Feasibility loop of Algorithm 3: drop the last J column while
   // min y_J <= 0 (and |J| > 1).  y_J only depends on the R22 triangle.  With
   // the positivity trick a J column enters with the sign of its w, and its y
-  // in [A -A] is that sign times the physical y.
+  // in [A -A] is that sign times the physical y.  The candidate lengths are
+  // tried at once, a warp each (back substitution with the columns scaled by
+  // their reciprocal diagonal: one FMA a step), and the fewest drops win;
+  // one warp that tried them in turn from global memory took 27 000 cycles
+  // at 32 columns without a drop.
   __device__ bool feasibility(const int* s_J) {
-    if (tm.rank == 0 && warp == 0) {
-      __shared__ double s_y[KM];
-      int k = kk, drops = 0;
-      for (;;) {
-        solve_r22(k, s_y);
-        __syncwarp();
-        double mn = INFINITY;
-        for (int t = lane; t < k; t += 32) {
-          const double sg = (sgn && ldcg(I.w + s_J[t]) < 0.0) ? -1.0 : 1.0;
-          mn = fmin(mn, sg * s_y[t]);
-        }
-        mn = warp_max(-mn);
-        mn = -mn;
-        if (!(mn <= 0.0) || k <= 1) break;
-        --k;
-        ++drops;
+    if (tm.rank == 0) {
+      constexpr int RS = KM + 1;
+      double* sR = dyn;             // column c at c RS
+      double* sp = sR + KM * RS;    // panel right-hand side
+      double* sri = sp + KM;        // reciprocal diagonal
+      __shared__ int s_fit;         // fewest drops found feasible
+      const int k0 = kk;
+      __syncthreads();
+      for (int c = warp; c < k0; c += NW) {
+        const double v0 = ldif(lane <= c, I.R22 + lane + c * KM), v1 = ldif(lane + 32 <= c, I.R22 + lane + 32 + c * KM);
+        sR[c * RS + lane] = v0;
+        sR[c * RS + lane + 32] = v1;
       }
-      for (int t = lane; t < k; t += 32) I.yJ[t] = s_y[t];
-      if (lane == 0) {
-        I.ctl[C_KP] = k;
-        I.ctl[C_DROPS] = drops;
+      if (tid < k0) sp[tid] = ldcg(I.pr + tid);
+      if (tid == 0) s_fit = k0;
+      __syncthreads();
+      if (tid < k0) sri[tid] = rcp_nr(sR[tid * RS + tid]);
+      __syncthreads();
+      for (int c = warp; c < k0; c += NW) {
+        const double ri = sri[c];
+        if (lane < c) sR[c * RS + lane] *= ri;
+        if (lane + 32 < c) sR[c * RS + lane + 32] *= ri;
+      }
+      __syncthreads();
+      for (int base = 0; base < k0; base += NW) {
+        const int d = base + warp, k = k0 - d;
+        double y0 = 0.0, y1 = 0.0;
+        if (k >= 1) {
+          double a0 = (lane < k) ? sp[lane] : 0.0, a1 = (lane + 32 < k) ? sp[lane + 32] : 0.0;
+          for (int j = k - 1; j >= 32; --j) {
+            const double aj = __shfl_sync(0xffffffffu, a1, j - 32);
+            a0 = fma(-sR[j * RS + lane], aj, a0);
+            if (lane + 32 < j) a1 = fma(-sR[j * RS + lane + 32], aj, a1);
+          }
+          for (int j = min(k, 32) - 1; j >= 0; --j) {
+            const double aj = __shfl_sync(0xffffffffu, a0, j);
+            if (lane < j) a0 = fma(-sR[j * RS + lane], aj, a0);
+          }
+          double mn = INFINITY;
+          if (lane < k) {
+            y0 = a0 * sri[lane];
+            mn = (sgn && ldcg(I.w + s_J[lane]) < 0.0) ? -y0 : y0;
+          }
+          if (lane + 32 < k) {
+            y1 = a1 * sri[lane + 32];
+            mn = fmin(mn, (sgn && ldcg(I.w + s_J[lane + 32]) < 0.0) ? -y1 : y1);
+          }
+          mn = -warp_max(-mn);
+          if ((!(mn <= 0.0) || k <= 1) && lane == 0) atomicMin(&s_fit, d);
+        }
+        __syncthreads();
+        const int fit = s_fit;
+        if (fit < base + NW) {
+          if (d == fit) {
+            if (lane < k) I.yJ[lane] = y0;
+            if (lane + 32 < k) I.yJ[lane + 32] = y1;
+            if (lane == 0) {
+              I.ctl[C_KP] = k;
+              I.ctl[C_DROPS] = fit;
+            }
+          }
+          break;
+        }
       }
     }
     if (!sync()) return false;
@@ -1185,7 +1226,7 @@ struct Engine {
   // the flag-pipelined solve, everything else the blocked solve.
   __device__ bool trsv(int np) {
     if (np <= 0) return true;
-    flops(cur_phase < 0 ? PH_SOLVE : cur_phase, (double)np * np);
+    flops(cur_phase < 0 ? PH_SOLVE : cur_phase, (long long)np * np);
     if (I.Dinv && tm.size >= 2 && np > 2 * TB) return trsv_pipelined(np);
     return trsv_blocked(np);
   }
@@ -1663,7 +1704,7 @@ struct Engine {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int c = (w0 + k * NW) * 32 + lane;
-        pv[k] = (w0 + k * NW < nwd && c < I.n) ? ldcg(I.pos + c) : 0;
+        pv[k] = ldif(w0 + k * NW < nwd && c < I.n, I.pos + c);
       }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -1677,45 +1718,36 @@ struct Engine {
       }
     }
     __syncthreads();
+    // exclusive prefix of the words' counts in s_jb, the total in s_nl
     if (warp == 0) {
-      int nz = 0;
-      for (int w0 = 0; w0 < nwd; w0 += 32) {
-        int cnt = (w0 + lane < nwd) ? __popc(s_zb[w0 + lane]) : 0;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        nz += cnt;
-      }
-      int lo, hi;
-      split(nz + (with_b ? 1 : 0), tm.size, tm.rank, lo, hi);
       int run = 0;
-      for (int w0 = 0; w0 < nwd && run < hi; w0 += 32) {
-        const unsigned bits = (w0 + lane < nwd) ? s_zb[w0 + lane] : 0u;
-        const int cnt = __popc(bits);
+      for (int w0 = 0; w0 < nwd; w0 += 32) {
+        const int cnt = (w0 + lane < nwd) ? __popc(s_zb[w0 + lane]) : 0;
         int inc = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int y = __shfl_up_sync(0xffffffffu, inc, o);
           if (lane >= o) inc += y;
         }
-        int r = run + inc - cnt;  // rank of this word's first Z column
-        if (r < hi && r + cnt > lo) {
-          unsigned bb = bits;
-          while (bb) {
-            const int bit = __ffs(bb) - 1;
-            bb &= bb - 1;
-            if (r >= lo && r < hi) s_list[r - lo] = (w0 + lane) * 32 + bit;
-            ++r;
-          }
-        }
+        if (w0 + lane < nwd) s_jb[w0 + lane] = (unsigned)(run + inc - cnt);
         run += __shfl_sync(0xffffffffu, inc, 31);
       }
-      if (lane == 0) {
-        if (with_b && nz >= lo && nz < hi) s_list[nz - lo] = -1;
-        s_nl = hi - lo;
-      }
+      if (lane == 0) s_nl = run;
     }
     __syncthreads();
-    return s_nl;
+    const int nz = s_nl;
+    int lo, hi;
+    split(nz + (with_b ? 1 : 0), tm.size, tm.rank, lo, hi);
+    for (int wd = warp; wd < nwd; wd += NW) {
+      const int r0 = (int)s_jb[wd];
+      const unsigned bits = s_zb[wd];
+      if (r0 >= hi || r0 + __popc(bits) <= lo) continue;
+      const int r = r0 + __popc(bits & ((1u << lane) - 1u));
+      if (((bits >> lane) & 1u) && r >= lo && r < hi) s_list[r - lo] = wd * 32 + lane;
+    }
+    if (tid == 0 && with_b && nz >= lo && nz < hi) s_list[nz - lo] = -1;
+    __syncthreads();
+    return hi - lo;
   }
 
   // Operands of one tensor-core commit batch (see commit()).
@@ -1742,7 +1774,8 @@ struct Engine {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int t = lane + 32 * h;
-        if (t < kp) sV[rr * VS + t] = (rg > t) ? ldcg(I.V + (size_t)rg * KM + t) : (rg == t) ? s_vt[t] : 0.0;
+        const double v = ldif(t < kp && rg > t, I.V + (size_t)rg * KM + t);
+        if (t < kp) sV[rr * VS + t] = (rg == t) ? s_vt[t] : v;
       }
     }
   }
@@ -2339,7 +2372,8 @@ struct Engine {
     if (tid == 0) s_guard = 0;
     for (int e = tid; e < r0d * kp; e += NT) {
       const int r = e / kp, t = e - r * kp;
-      sTV[e] = (r > t) ? ldcg(I.V + (size_t)r * KM + t) : (r == t) ? cs.s_vt[t] : 0.0;
+      const double v = ldif(r > t, I.V + (size_t)r * KM + t);
+      sTV[e] = (r == t) ? cs.s_vt[t] : v;
     }
     for (int e = tid; e < r0d * NB; e += NT) {
       const int c = e / r0d, r = e - c * r0d;
@@ -2753,16 +2787,14 @@ struct Engine {
   // and column norms of C).
   __device__ __forceinline__ bool commit(const int* s_J) {
     const int L = I.m - nP;
-    flops(PH_COMMIT, 4.0 * kp * (double)L * (double)(I.n - nP - kp + 1) + 2.0 * (double)L * (I.n - nP - kp));
+    flops(PH_COMMIT, 4ll * kp * L * (I.n - nP - kp + 1) + 2ll * L * (I.n - nP - kp));
     // (a) R columns of the new positions (free slots rslot[nP..nP+kp))
     {
-      const int gt = tm.rank * NT + tid, nt = tm.size * NT;
-      const int tot = (nP + KM) * kp;
-      for (int e = gt; e < tot; e += nt) {
-        const int t = e / (nP + KM), row = e - t * (nP + KM);
-        const int slot = ldcg(I.rslot + nP + t);
-        if (row < nP) Rcol(slot)[row] = ldcg(Wcol(s_J[t]) + row);
-        else if (row - nP <= t) Rcol(slot)[row] = ldcg(I.R22 + (row - nP) + t * KM);
+      const int nrb = (nP + kp + 31) >> 5;  // a warp takes 32 rows of a column
+      for (int un = tm.rank * NW + warp; un < kp * nrb; un += tm.size * NW) {
+        const int t = un / nrb, row = (un - t * nrb) * 32 + lane;
+        if (row <= nP + t)
+          Rcol(ldcg(I.rslot + nP + t))[row] = ldcg(row < nP ? Wcol(s_J[t]) + row : I.R22 + (row - nP) + t * KM);
       }
       if (tm.rank == 0 && tid < kp) {
         I.order[nP + tid] = s_J[tid];
@@ -2880,8 +2912,7 @@ struct Engine {
       // any y_P <= 0 ?  (with the positivity trick: y of the signed column)
       int neg = 0;
       for (int p = tid; p < nP; p += NT) neg |= (pos_sign(p) * ldcg(I.yP + p) <= 0.0);
-      neg = block_sum_int(neg, shi);
-      if (!neg) return true;
+      if (!__syncthreads_or(neg)) return true;
       if (steps > nP + 1) {
         status = LHDM_ERR_MAX_ITER;
         return true;
@@ -2960,8 +2991,8 @@ struct Engine {
     const int np = nP;
     inv_valid = min(inv_valid, q);
     const int nrot = np - 1 - q;
-    flops(PH_CHAIN, 3.0 * (double)nrot * (nrot + 1));
-    flops(PH_ZROT, 6.0 * (double)nrot * (double)(I.n - np + 2));
+    flops(PH_CHAIN, 3ll * nrot * (nrot + 1));
+    flops(PH_ZROT, 6ll * nrot * (I.n - np + 2));
     if (tm.rank == 0) {
       // the removed column re-enters Z in trailing form: W(:, c) = [R(0:q, slot); 0]
       const int c = ldcg(I.order + q);
@@ -3750,9 +3781,14 @@ struct Engine {
       s_acc[warp][lane] = acc + acc2;
       __syncthreads();
       if (warp == 0 && row < I.m) {
-        double s = 0.0;
-        for (int k = 0; k < NW; ++k) s += s_acc[k][lane];
-        const double rv = __ldg(I.b + row) - s;
+        double t[NW];
+#pragma unroll
+        for (int k = 0; k < NW; ++k) t[k] = s_acc[k][lane];
+#pragma unroll
+        for (int o = NW / 2; o; o >>= 1)
+#pragma unroll
+          for (int k = 0; k < o; ++k) t[k] += t[k + o];
+        const double rv = __ldg(I.b + row) - t[0];
         I.r[row] = rv;
         rs = fma(rv, rv, rs);
       }
@@ -3761,9 +3797,10 @@ struct Engine {
     // x = y on P
     const int gt = tm.rank * NT + tid, nt = tm.size * NT;
     for (int p = gt; p < nP; p += nt) I.xP[p] = ldcg(I.yP + p);
-    __shared__ double sh[32];
-    rs = block_sum(rs, sh);
-    if (tid == 0) I.part[(size_t)tm.rank * PW + P_RS] = rs;
+    if (warp == 0) {  // only warp 0 holds squares
+      rs = warp_sum(rs);
+      if (lane == 0) I.part[(size_t)tm.rank * PW + P_RS] = rs;
+    }
   }
 
   // w = A^T r on Z (w_P = 0) and the O1 partial.  The Z columns are split
@@ -3790,6 +3827,7 @@ struct Engine {
     int* s_zl = reinterpret_cast<int*>(dyn + (r_in_smem ? m : 0));
     unsigned* scr = reinterpret_cast<unsigned*>(s_zl + CAND_LOCAL_MAX + 2);
     __shared__ double s_pp[NW][2];  // partial sums of a warp's first and last column
+    __shared__ int s_kr[NW][2];     // those columns (none: 0, -1)
     const int nl = z_share(s_zl, scr, nullptr, 0, false);
     if (r_in_smem)
       for (int i = tid; i < m; i += NT) s_r[i] = ldcg(I.r + i);
@@ -3798,8 +3836,23 @@ struct Engine {
     const long long E = (long long)nl * m;
     {
       const long long e0 = E * warp / NW, e1 = E * (warp + 1) / NW;
+      if (lane == 0) {
+        s_kr[warp][0] = 0;
+        s_kr[warp][1] = -1;
+      }
       if (e0 < e1) {
-        const int kf = (int)(e0 / m), kl = (int)((e1 - 1) / m);
+        int kf, kl;
+        if (E < (1ll << 31)) {
+          kf = (int)((unsigned)e0 / (unsigned)m);
+          kl = (int)((unsigned)(e1 - 1) / (unsigned)m);
+        } else {
+          kf = (int)(e0 / m);
+          kl = (int)((e1 - 1) / m);
+        }
+        if (lane == 0) {
+          s_kr[warp][0] = kf;
+          s_kr[warp][1] = kl;
+        }
         for (int k = kf; k <= kl; ++k) {
           const int i0 = (k == kf) ? (int)(e0 - (long long)k * m) : 0;
           const int i1 = (k == kl) ? (int)(e1 - (long long)k * m) : m;
@@ -3831,18 +3884,13 @@ struct Engine {
     }
     __syncthreads();
     for (int k = tid; k < nl; k += NT) {
-      const long long cs = (long long)k * m, ce = cs + m;
       double sum = 0.0;
-      bool direct = false;
+      bool direct = false;  // written by the warp that has all of it
       for (int w = 0; w < NW; ++w) {
-        const long long a0 = E * w / NW, a1 = E * (w + 1) / NW;
-        if (a0 >= a1 || a1 <= cs || a0 >= ce) continue;
-        const int kf = (int)(a0 / m), kl = (int)((a1 - 1) / m);
-        if (k != kf && k != kl) {
-          direct = true;  // written by warp w
-          break;
-        }
-        sum += (k == kf) ? s_pp[w][0] : s_pp[w][1];
+        const int kf = s_kr[w][0], kl = s_kr[w][1];
+        if (k < kf || k > kl) continue;
+        direct |= k != kf && k != kl;
+        sum += s_pp[w][k == kf ? 0 : 1];
       }
       if (!direct) I.w[s_zl[k]] = sum;
     }
@@ -3925,8 +3973,8 @@ struct Engine {
       if (I.phase_ns) {
         phase(-1);
         for (int i = 0; i < NPHASE; ++i) {
-          I.phase_ns[i] = phf[i];
-          I.phase_ns[NPHASE + i] = phf[NPHASE + i];
+          I.phase_ns[i] = (double)phf[i];
+          I.phase_ns[NPHASE + i] = (double)phf[NPHASE + i];
         }
       }
     }
@@ -3937,7 +3985,7 @@ struct Engine {
   __device__ __forceinline__ void run() {
     phase(PH_SETUP);
     setup();
-    flops(PH_SETUP, 4.0 * (double)I.m * I.n);
+    flops(PH_SETUP, 4ll * I.m * I.n);
     if (!sync()) return fail_out();
     o1_reduce(true);
     tol_w = (I.prm.tol_w >= 0.0) ? I.prm.tol_w
@@ -3988,11 +4036,18 @@ struct Engine {
         const int gt = tm.rank * NT + tid, nt = tm.size * NT;
         for (int p = gt; p < nP; p += nt) {
           double s = ldcg(I.bt + p);
-          for (int t = 0; t < kp; ++t) s = fma(-ldcg(Wcol(s_J[t]) + p), s_yj[t], s);
+          for (int t0 = 0; t0 < kp; t0 += 8) {
+            double v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = ldif(t0 + j < kp, Wcol(s_J[min(t0 + j, kp - 1)]) + p);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (t0 + j < kp) s = fma(-v[j], s_yj[t0 + j], s);
+          }
           I.rhs[p] = s;
         }
       }
-      flops(PH_SOLVE, 2.0 * nP * (double)kp + (double)kk * kk);
+      flops(PH_SOLVE, 2ll * nP * kp + (long long)kk * kk);
       if (!sync()) return fail_out();
       if (!trsv(nP)) return fail_out();
       phase(PH_COMMIT);
@@ -4003,11 +4058,11 @@ struct Engine {
       if (!inner_loop()) return fail_out();
       if (status != LHDM_OK) break;
       phase(PH_RESID);
-      flops(PH_RESID, 2.0 * (double)I.m * nP);
+      flops(PH_RESID, 2ll * I.m * nP);
       residual();
       if (!sync()) return fail_out();
       phase(PH_DUAL);
-      flops(PH_DUAL, 2.0 * (double)I.m * (double)(I.n - nP));
+      flops(PH_DUAL, 2ll * I.m * (I.n - nP));
       dual();
       if (!sync()) return fail_out();
       if (I.trace && tm.rank == 0 && tid == 0 && n_outer < I.trace_cap) {
