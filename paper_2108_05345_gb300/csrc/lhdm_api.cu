@@ -27,6 +27,7 @@ struct lhdm_ctx {
   double* dscr = nullptr;
   int* iscr = nullptr;
   double* R = nullptr;
+  double* Rinv = nullptr;  // part of R's allocation; null: the solve substitutes
   int* rslot = nullptr;
   int* order = nullptr;
   double* xP = nullptr;
@@ -190,7 +191,16 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
   cudaError_t e = cudaSuccess;
   e = cudaMalloc(&c->dscr, c->L.dtotal * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->iscr, c->L.itotal * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->R, (size_t)c->ldr * c->cap * sizeof(double));
+  // R and, behind it, its kept inverse (without it where memory is short)
+  const size_t nR = (size_t)c->ldr * c->cap;
+  if (e == cudaSuccess) {
+    if (cudaMalloc(&c->R, 2 * nR * sizeof(double)) == cudaSuccess) {
+      c->Rinv = c->R + nR;
+    } else {
+      cudaGetLastError();
+      e = cudaMalloc(&c->R, nR * sizeof(double));
+    }
+  }
   if (e == cudaSuccess) e = cudaMalloc(&c->rslot, (size_t)c->cap * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->order, (size_t)c->cap * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->xP, (size_t)c->cap * sizeof(double));
@@ -280,6 +290,7 @@ int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, 
   I.passive_out = passive;
   I.prm = to_dev(p);
   fill_ctx_inst(c, I);
+  I.Rinv = c->Rinv;
   I.bar_extra = c->stall_next ? 1 : 0;
   c->stall_next = false;
   c->have_state = false;

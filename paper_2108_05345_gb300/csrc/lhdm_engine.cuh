@@ -88,11 +88,13 @@ struct Inst {
   double* xP;
   double* r;
   int* nP_out;
+  double* Rinv;   // inverse of R, row of position p in slot rslot[p] (ld ldr; null: not kept)
   // scratch
   double* W;
   double* bt;
   double* yP;
   double* rhs;
+  double* rres;   // cap: residual of a corrected solve
   double* w;
   double* u;
   double* anorm;
@@ -133,13 +135,15 @@ struct Inst {
   int bar_extra;              // failure-detection test: arrivals the grid barrier
                               // expects beyond the grid (0 in every normal solve)
   int guard_force;            // test aid: 1 sends every tensor-core commit batch to
-                              // FP64 as the accuracy guard would (0 in normal solves)
+                              // FP64 as the accuracy guard would, and fails the kept
+                          // inverse's residual test (0 in normal solves)
   DevParams prm;
 };
 
 // control words (ctl[])
 enum { C_KP = 0, C_DROPS, C_CAND, C_NROT, C_NRUN, C_READY, C_STATUS, C_ERR, C_KK, C_NFLIP,
-       C_GUARD1 }; // commit batches the accuracy guard handed to the FP64 path
+       C_GUARD1,  // commit batches the accuracy guard handed to the FP64 path
+       C_INV };   // last corrected solve whose residual test failed
 
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }

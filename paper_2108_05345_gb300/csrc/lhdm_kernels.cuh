@@ -38,7 +38,7 @@ struct BatchItem {
 
 // Offsets of one team's scratch inside a double region and an int region.
 struct ScratchLayout {
-  size_t W, bt, yP, rhs, w, u, anorm, V, vtop, beta, T, R22, Gm, yJ, pr, part, pacc, candw, rotc, rots, apu;
+  size_t W, bt, yP, rhs, rres, w, u, anorm, V, vtop, beta, T, R22, Gm, yJ, pr, part, pacc, candw, rotc, rots, apu;
   size_t Dinv, accb;  // pipelined triangular solve (teams of more than one CTA)
   size_t dtotal;
   size_t Vd;  // reflector digits of the tensor-core commit
@@ -61,6 +61,7 @@ inline ScratchLayout make_layout(int max_m, int max_n, int team) {
   L.bt = take(m);
   L.yP = take(cap);
   L.rhs = take(std::max(m, cap));
+  L.rres = take(team > 1 ? cap : 1);
   L.w = take(n);
   L.u = take(n);
   L.anorm = take(n);
@@ -106,6 +107,8 @@ inline __host__ __device__ void bind_scratch(Inst& I, const ScratchLayout& L, do
   I.bt = d + L.bt;
   I.yP = d + L.yP;
   I.rhs = d + L.rhs;
+  I.rres = d + L.rres;
+  I.Rinv = nullptr;
   I.w = d + L.w;
   I.u = d + L.u;
   I.anorm = d + L.anorm;

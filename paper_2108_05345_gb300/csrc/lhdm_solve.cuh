@@ -46,6 +46,9 @@ struct Engine {
   int kdm = 0, removed = 0, inner_step = 0;
   int inv_valid = 0;  // positions whose diagonal-block inverse column is current
   int tepoch = 0;     // pipelined-solve calls in this launch (flag values)
+  int iepoch = 0;     // corrected solves in this launch (flag values)
+  bool inv_on = false;  // R^{-1} may be kept
+  int inv_n = 0;        // leading positions whose inverse is current
   int sgn = 0;        // I.prm.mode: 0 plain NNLS, 1 positivity trick, 2 with sign flip
   int nx = 0;         // columns of the problem solved: n, or 2n for [A -A]
   int n_flip = 0;     // sign flips (mode 2)
@@ -64,6 +67,7 @@ struct Engine {
     warp = tid >> 5;
     sgn = I.prm.mode;
     nx = sgn ? 2 * I.n : I.n;
+    inv_on = I.Rinv != nullptr;
     __shared__ long long s_phf[2 * NPHASE];
     phf = s_phf;
     if (tid == 0)
@@ -1685,6 +1689,287 @@ struct Engine {
 
 
 
+  // ------------------------------------------------------------ explicit inverse
+  // The whole-GPU solve can keep R^{-1} (row p of position p, in slot rslot[p];
+  // zeros left of the diagonal; inv_n leading positions are current), so that
+  // a solve with R is products that every warp of the GPU shares instead of a
+  // chain over 64-row blocks (about 8 000 cycles a block): y = R^{-1} rhs, one
+  // correction y += R^{-1} (rhs - R y), three barriers, about 25 000 cycles at
+  // any size up to 2048.  Measured per solve: inner steps of the 4096 x 2048
+  // instance 88 -> 23 us, of the conditioned 2048 x 1024 one 41 -> 12 us,
+  // one-column steps at 2048 x 1024 31 -> 18 us.
+  //  append: with S = R^{-1} R12 the new columns are -S R22^{-1}, the new rows
+  //    R22^{-1}, and y_P = R^{-1} Q^T b - S y_J falls out of the same pass.
+  //  downdate: R~ E = G^T R_new gives R_new^{-1} = E^T R^{-1} G^T: the rotations
+  //    that act on R's rows act on the columns of R^{-1} (rotate_columns).
+  // An append costs nP^2 k / 2 FMAs over the GPU, so the inverse is made when
+  // an inner step first solves with more than INV_MIN positions (below, the
+  // substitution is one or two blocks) or when k <= 3, and follows from there.
+  // Accuracy: the correction's residual is tested row by row against the
+  // row's largest |R| |y|: one product with the inverse leaves about
+  // |I - R R^{-1}| of it, the second the square of that, so 2^-26 guarantees
+  // rounding level.  Where a row misses it (R too ill-conditioned for an
+  // explicit inverse) the solve is done by substitution and the inverse is
+  // given up for the rest.
+  static constexpr int INV_MIN = 2 * TB, INV_ROWS = 3072;
+  static constexpr int INV_BITS = 26;
+  __device__ __forceinline__ double* Irow(int p) const { return I.Rinv + (size_t)ldcg(I.rslot + p) * I.ldr; }
+
+  // yP (+)= R^{-1} v on positions [0, np), a warp per row.
+  __device__ void inv_product(int np, const double* v, bool add) {
+    for (int p = tm.rank + tm.size * warp; p < np; p += tm.size * NW) {
+      const double* row = Irow(p);
+      double a0 = 0.0, a1 = 0.0;
+      for (int j0 = p & ~31; j0 < np; j0 += 256) {
+        double rv[8], xv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = min(j0 + 32 * u + lane, np - 1);
+          rv[u] = ldcg(row + j);
+          xv[u] = ldcg(v + j);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          if (j0 + 32 * u + lane < np) a0 = fma(rv[u], xv[u], a0);
+          if (j0 + 32 * u + 32 + lane < np) a1 = fma(rv[u + 1], xv[u + 1], a1);
+        }
+      }
+      const double t = warp_sum(a0 + a1);
+      if (lane == 0) I.yP[p] = add ? ldcg(I.yP + p) + t : t;
+    }
+  }
+
+  // Sums over j of R^{-1}(p, j) col_a(j) for the nt <= NA columns src[0 ..]
+  // (and of R^{-1}(p, j) (Q^T b)_j) over the first c0 positions, by one warp,
+  // lanes over j; they land in out[a] (and *zout).
+  template <int NA, int U>
+  __device__ __forceinline__ void inv_row_products(int p, int c0, const double* const* src, int nt, double* out,
+                                                   double* zout) {
+    const double* row = Irow(p);
+    double acc[NA], z = 0.0;
+    const double* wp[NA];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      acc[a] = 0.0;
+      wp[a] = src[min(a, nt - 1)];
+    }
+    for (int j0 = p & ~31; j0 < c0; j0 += 32 * U) {
+      double rv[U], wv[U][NA], bv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = min(j0 + 32 * u + lane, c0 - 1);
+        rv[u] = ldcg(row + j);
+        bv[u] = zout ? ldcg(I.bt + j) : 0.0;
+#pragma unroll
+        for (int a = 0; a < NA; ++a) wv[u][a] = ldcg(wp[a] + j);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const double r = (j0 + 32 * u + lane < c0) ? rv[u] : 0.0;
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+          if (a < nt) acc[a] = fma(r, wv[u][a], acc[a]);
+        if (zout) z = fma(r, bv[u], z);
+      }
+    }
+    if constexpr (NA == 8) {
+      // transposing sum: after three halvings lane l holds value l >> 2 over
+      // four lanes' shares; nine additions for eight sums
+#pragma unroll
+      for (int w = 4, o = 16; w >= 1; w >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int a = 0; a < w; ++a) {
+          const double keep = up ? acc[a + w] : acc[a], give = up ? acc[a] : acc[a + w];
+          acc[a] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      }
+      double v = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      if ((lane & 3) == 0 && (lane >> 2) < nt) out[lane >> 2] = v;
+    } else {
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        const double v = warp_sum(acc[a]);
+        if (lane == 0 && a < nt) out[a] = v;
+      }
+    }
+    if (zout) {
+      z = warp_sum(z);
+      if (lane == 0) *zout = z;
+    }
+  }
+
+  // Extends the inverse from c0 to c0 + k positions (k <= KM; a barrier must
+  // follow).  fresh: the columns are J[0:k] of the append under way (R12 in W,
+  // the triangle in R22), and rows p < c0 also get y_P and rhs for the solve
+  // that goes with it; else they are R's columns c0 .. c0 + k - 1.  Rows go
+  // round over the CTAs, sixteen at a time; a CTA's (row, eight columns) units
+  // go over its warps.
+  __device__ void inv_extend(int c0, int k, bool fresh, const int* s_J, const double* s_yj) {
+    constexpr int RS = KM + 1;
+    double* sR = dyn;              // triangle(s, t) / triangle(s, s) at s RS + t, s < t
+    double* sri = sR + KM * RS;    // reciprocal diagonal
+    double* sS = sri + KM;         // NW x RS: S of the CTA's rows
+    double* sz = sS + NW * RS;     // NW
+    __shared__ const double* s_src[KM];  // rows 0 .. c0 + of the new columns
+    __syncthreads();
+    if (tid < k) s_src[tid] = fresh ? Wcol(s_J[tid]) : Rcol(ldcg(I.rslot + c0 + tid));
+    __syncthreads();
+    if (tid < k) sri[tid] = rcp_nr(ldcg(fresh ? I.R22 + tid + tid * KM : s_src[tid] + c0 + tid));
+    __syncthreads();
+    for (int t = warp; t < k; t += NW) {  // column t of the triangle
+      const double* col = fresh ? I.R22 + t * KM : s_src[t] + c0;
+      const double v0 = ldif(lane < t, col + lane), v1 = ldif(lane + 32 < t, col + lane + 32);
+      if (lane < k) sR[lane * RS + t] = v0 * sri[lane];
+      if (lane + 32 < k) sR[(lane + 32) * RS + t] = v1 * sri[lane + 32];
+    }
+    const int rows = c0 + k, ngrp = k <= 3 ? 1 : (k + 7) >> 3;
+    for (int base = 0; tm.rank + tm.size * base < rows; base += NW) {
+      const int left = c0 - tm.rank - tm.size * base;  // rows below c0 of this batch
+      const int nrow = left <= 0 ? 0 : min(NW, (left + tm.size - 1) / tm.size);
+      __syncthreads();
+      for (int un = warp; un < nrow * ngrp; un += NW) {
+        const int i = un / ngrp, g = un - i * ngrp, p = tm.rank + tm.size * (base + i);
+        double* zo = (fresh && g == 0) ? sz + i : nullptr;
+        if (k <= 3) inv_row_products<3, 4>(p, c0, s_src, k, sS + i * RS, zo);
+        else inv_row_products<8, 2>(p, c0, s_src + 8 * g, min(8, k - 8 * g), sS + i * RS + 8 * g, zo);
+      }
+      __syncthreads();
+      const int p = tm.rank + tm.size * (base + warp);
+      if (p < rows) {
+        double* row = Irow(p);
+        double a0 = 0.0, a1 = 0.0;
+        if (p < c0) {
+          const double s0 = (lane < k) ? sS[warp * RS + lane] : 0.0, s1 = (lane + 32 < k) ? sS[warp * RS + lane + 32] : 0.0;
+          if (fresh) {
+            const double y0 = (lane < k) ? s_yj[lane] : 0.0, y1 = (lane + 32 < k) ? s_yj[lane + 32] : 0.0;
+            const double w0 = ldif(lane < k, s_src[min(lane, k - 1)] + p);
+            const double w1 = ldif(lane + 32 < k, s_src[min(lane + 32, k - 1)] + p);
+            const double ys = warp_sum(fma(s0, y0, s1 * y1)), rs = warp_sum(fma(w0, y0, w1 * y1));
+            if (lane == 0) {
+              I.yP[p] = sz[warp] - ys;
+              I.rhs[p] = ldcg(I.bt + p) - rs;
+            }
+          }
+          a0 = -s0;
+          a1 = -s1;
+        } else {
+          for (int j = lane; j < c0; j += 32) row[j] = 0.0;
+          a0 = (lane == p - c0) ? 1.0 : 0.0;
+          a1 = (lane + 32 == p - c0) ? 1.0 : 0.0;
+        }
+        // x times the triangle = a, columns left to right
+        for (int q = 0; q < min(k, 32); ++q) {
+          const double aq = __shfl_sync(0xffffffffu, a0, q);
+          if (lane > q && lane < k) a0 = fma(-sR[q * RS + lane], aq, a0);
+          if (lane + 32 < k) a1 = fma(-sR[q * RS + lane + 32], aq, a1);
+        }
+        for (int q = 32; q < k; ++q) {
+          const double aq = __shfl_sync(0xffffffffu, a1, q - 32);
+          if (lane + 32 > q && lane + 32 < k) a1 = fma(-sR[q * RS + lane + 32], aq, a1);
+        }
+        if (lane < k) row[c0 + lane] = a0 * sri[lane];
+        if (lane + 32 < k) row[c0 + lane + 32] = a1 * sri[lane + 32];
+      }
+    }
+  }
+
+  // Residual rhs - R yP on rows [0, np) into rres, eight rows per CTA and
+  // pass (lanes: 8 rows x 4 columns), with the accuracy test.
+  __device__ void inv_residual(int np, int ep) {
+    double* sy = dyn;                                    // np
+    int* ss = reinterpret_cast<int*>(dyn + np);          // np
+    double* sa = dyn + np + (np + 1) / 2;                // NW x 8
+    int* sf = reinterpret_cast<int*>(sa + NW * 8);       // NW x 8
+    if (tm.rank * 8 >= np) return;
+    __syncthreads();
+    const int first = tm.rank * 8;
+    for (int c = first + tid; c < np; c += NT) {
+      sy[c] = ldcg(I.yP + c);
+      ss[c] = ldcg(I.rslot + c);
+    }
+    __syncthreads();
+    const int row = lane & 7, cg = lane >> 3;
+    for (int p0 = first; p0 < np; p0 += tm.size * 8) {
+      double a = 0.0;
+      int f = -8000;  // largest exponent of |R| |y| (a conversion to float is an FP64 instruction)
+      const int r = min(p0 + row, np - 1);
+      for (int c0 = p0 + warp * 4 + cg; c0 < np; c0 += 8 * 4 * NW) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = ldcg(Rcol(ss[min(c0 + u * 4 * NW, np - 1)]) + r);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int c = c0 + u * 4 * NW;
+          if (c < np && c >= r) {
+            const double y = sy[c];
+            a = fma(v[u], y, a);
+            f = max(f, ebound(v[u]) + ebound(y));
+          }
+        }
+      }
+      a += __shfl_xor_sync(0xffffffffu, a, 8);
+      a += __shfl_xor_sync(0xffffffffu, a, 16);
+      f = max(f, __shfl_xor_sync(0xffffffffu, f, 8));
+      f = max(f, __shfl_xor_sync(0xffffffffu, f, 16));
+      if (lane < 8) {
+        sa[warp * 8 + lane] = a;
+        sf[warp * 8 + lane] = f;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        double t = 0.0;
+        int g = -8000;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          t += sa[(4 * cg + k) * 8 + row];
+          g = max(g, sf[(4 * cg + k) * 8 + row]);
+        }
+        t += __shfl_xor_sync(0xffffffffu, t, 8);
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        g = max(g, __shfl_xor_sync(0xffffffffu, g, 8));
+        g = max(g, __shfl_xor_sync(0xffffffffu, g, 16));
+        if (lane < 8 && p0 + lane < np) {
+          const double d = ldcg(I.rhs + p0 + lane) - t;
+          I.rres[p0 + lane] = d;
+          // |d| <= 2^-INV_BITS times the largest term (at least 2^(g - 2)); a
+          // term that is not finite fails
+          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || I.guard_force) I.ctl[C_INV] = ep;
+        }
+      }
+      __syncthreads();
+    }
+  }
+
+  // R y = rhs on [0, np) with yP already R^{-1} rhs (a barrier must have
+  // followed): the correction, or the substitution where the test fails.
+  __device__ bool inv_correct(int np) {
+    const int ep = ++iepoch;
+    inv_residual(np, ep);
+    if (!sync()) return false;
+    if (ldcg(I.ctl + C_INV) == ep) {
+      inv_on = false;
+      return trsv(np);
+    }
+    inv_product(np, I.rres, true);
+    return sync();
+  }
+  // R y = rhs on [0, np) (the inner step's solve)
+  __device__ bool solve_tri(int np) {
+    if (!inv_on || np > INV_ROWS || (np <= INV_MIN && inv_n < np)) return trsv(np);
+    while (inv_n < np) {
+      const int k = min(32, np - inv_n);
+      inv_extend(inv_n, k, false, nullptr, nullptr);
+      if (!sync()) return false;
+      inv_n += k;
+    }
+    flops(cur_phase < 0 ? PH_SOLVE : cur_phase, (long long)np * np);
+    inv_product(np, I.rhs, false);
+    if (!sync()) return false;
+    return inv_correct(np);
+  }
+
   // This CTA's share of the Z columns: the columns with pos < 0 that are not
   // in J[0:nj] are numbered in column order (with b = -1 appended last when
   // with_b) and split evenly over the team, so every CTA gets floor or ceil
@@ -2977,7 +3262,7 @@ struct Engine {
       }
       // re-solve: rhs = (Q^T b)[0:nP] was written by the owner of b
       phase(PH_ITRSV);
-      if (!trsv(nP)) return false;
+      if (!solve_tri(nP)) return false;
       phase(PH_INNER);
     }
   }
@@ -3418,6 +3703,7 @@ struct Engine {
     phase(PH_ZROT);
     nP = np - 1;
     if (!follow) rotate_columns(q, np, nrot, 0, false);
+    inv_n = (inv_n == np) ? np - 1 : min(inv_n, q);
     const bool ok = sync();
     phase(PH_INNER);
     return ok;
@@ -3461,7 +3747,9 @@ struct Engine {
     // R columns round-robin over the ranks (the last positions, which take
     // the most rotations, land on different CTAs)
     const int nr_own = (zr < nrot) ? (nrot - zr + nzr - 1) / nzr : 0;
-    const int nunit = nz + nr_own;
+    // rows of R^{-1}, one position after another like R's columns
+    const int ni_own = (inv_n == np && zr < np - 1) ? (np - 1 - zr + nzr - 1) / nzr : 0;
+    const int nunit = nz + nr_own + ni_own;
     // the products for the chunk at stage offset t0 (one warp)
     auto chunk_products = [&](int t0, int ns) {
       const int cnt = min(32, ns - t0);
@@ -3496,12 +3784,19 @@ struct Engine {
       carry = __shfl_sync(0xffffffffu, incl, cnt - 1);
     };
     // unit k: its column, its rotation count from rb on, whether they end an
-    // R column's rotations
-    auto unit = [&](int k, int rb, int ns, double*& colp, int& nsu, bool& rlast) {
+    // R column's rotations, the first chunk that is not all zeros (row p of
+    // R^{-1} starts at column p)
+    auto unit = [&](int k, int rb, int ns, double*& colp, int& nsu, bool& rlast, int& ts) {
       nsu = ns;
       rlast = false;
+      ts = 0;
       if (k < nz) {
         colp = (k < s_nz) ? Wcol(s_zl[k]) : I.bt;
+      } else if (k >= nz + nr_own) {
+        const int p = zr + (k - nz - nr_own) * nzr;
+        colp = Irow(p);
+        ts = max(0, (max(0, p - q) & ~31) - rb);
+        if (ts >= ns) nsu = 0;
       } else {
         const int pr = q + zr + (k - nz) * nzr;  // R column at position pr
         colp = Rcol(ldcg(I.rslot + pr));
@@ -3548,7 +3843,8 @@ struct Engine {
         double* colp = I.bt;
         int nsu = 0;
         bool rlast = false;
-        if (k < ncol) unit(k, 0, nrot, colp, nsu, rlast);
+        int ts;
+        if (k < ncol) unit(k, 0, nrot, colp, nsu, rlast, ts);
         double carry = (nsu > 0) ? ldcg(colp + q) : 0.0;
         int gmax = nsu;
 #pragma unroll
@@ -3607,12 +3903,13 @@ struct Engine {
           double* colp;
           int nsu;
           bool rlast;
-          unit(k, rb, ns, colp, nsu, rlast);
+          int ts;
+          unit(k, rb, ns, colp, nsu, rlast, ts);
           if (nsu <= 0) continue;
-          double carry = ldcg(colp + q + rb);
+          double carry = ldcg(colp + q + rb + ts);
           // next chunk's column values are loaded before the scan of this one
-          double nbot = (lane < nsu) ? ldcg(colp + q + rb + 1 + lane) : 0.0;
-          for (int t0 = 0; t0 < nsu; t0 += 32) {
+          double nbot = (ts + lane < nsu) ? ldcg(colp + q + rb + ts + 1 + lane) : 0.0;
+          for (int t0 = ts; t0 < nsu; t0 += 32) {
             const double bot = nbot;
             nbot = (t0 + 32 + lane < nsu) ? ldcg(colp + q + rb + t0 + 33 + lane) : 0.0;
             chunk_apply(colp, rb, t0, min(32, nsu - t0), bot, carry);
@@ -3700,16 +3997,18 @@ struct Engine {
         double* colp;
         int nsu;
         bool rlast;
-        unit(k, 0, nrot, colp, nsu, rlast);
+        int ts;
+        unit(k, 0, nrot, colp, nsu, rlast, ts);
+        if (nsu <= 0) continue;
         // an R column waits for its own chain block's rotations: that block
         // read the column from global memory before generating them
-        if (k >= nz && !wait_avail((nsu - 1) / DB + 1)) {
+        if (k >= nz && k < nz + nr_own && !wait_avail((nsu - 1) / DB + 1)) {
           ok = false;
           break;
         }
-        double carry = ldcg(colp + q);
-        double nbot = (lane < nsu) ? ldcg(colp + q + 1 + lane) : 0.0;
-        for (int t0 = 0; t0 < nsu; t0 += 32) {
+        double carry = ldcg(colp + q + ts);
+        double nbot = (ts + lane < nsu) ? ldcg(colp + q + ts + 1 + lane) : 0.0;
+        for (int t0 = ts; t0 < nsu; t0 += 32) {
           if (!wait_avail(t0 / 32 + 1)) {
             ok = false;
             break;
@@ -4028,11 +4327,19 @@ struct Engine {
       phase(PH_FEAS);
       if (!feasibility(s_J)) return fail_out();
       phase(PH_SOLVE);
-      // y_P: rhs = (Q^T b)[0:nP] - R12 y_J, then back substitution
-      {
-        __shared__ double s_yj[KM];
-        if (tid < kp) s_yj[tid] = ldcg(I.yJ + tid);
-        __syncthreads();
+      // y_P: rhs = (Q^T b)[0:nP] - R12 y_J, then R y_P = rhs
+      __shared__ double s_yj[KM];
+      if (tid < kp) s_yj[tid] = ldcg(I.yJ + tid);
+      __syncthreads();
+      flops(PH_SOLVE, 2ll * nP * kp + (long long)kk * kk);
+      if (inv_on && inv_n == nP && nP + kp <= INV_ROWS && (kp <= 3 || nP > INV_MIN)) {
+        inv_extend(nP, kp, true, s_J, s_yj);
+        inv_n = nP + kp;
+        if (nP > 0) {
+          flops(PH_SOLVE, (long long)nP * nP);
+          if (!sync() || !inv_correct(nP)) return fail_out();
+        }
+      } else {
         const int gt = tm.rank * NT + tid, nt = tm.size * NT;
         for (int p = gt; p < nP; p += nt) {
           double s = ldcg(I.bt + p);
@@ -4046,10 +4353,9 @@ struct Engine {
           }
           I.rhs[p] = s;
         }
+        if (!sync()) return fail_out();
+        if (!trsv(nP)) return fail_out();
       }
-      flops(PH_SOLVE, 2ll * nP * kp + (long long)kk * kk);
-      if (!sync()) return fail_out();
-      if (!trsv(nP)) return fail_out();
       phase(PH_COMMIT);
       if (!commit(s_J)) return fail_out();
       phase(PH_INNER);
