@@ -135,15 +135,16 @@ struct Inst {
   int bar_extra;              // failure-detection test: arrivals the grid barrier
                               // expects beyond the grid (0 in every normal solve)
   int guard_force;            // test aid: 1 sends every tensor-core commit batch to
-                              // FP64 as the accuracy guard would, and fails the kept
-                          // inverse's residual test (0 in normal solves)
+                              // FP64 as the accuracy guard would, and fails the tests
+                          // of the kept inverse in inner steps (0 in normal solves)
   DevParams prm;
 };
 
 // control words (ctl[])
 enum { C_KP = 0, C_DROPS, C_CAND, C_NROT, C_NRUN, C_READY, C_STATUS, C_ERR, C_KK, C_NFLIP,
        C_GUARD1,  // commit batches the accuracy guard handed to the FP64 path
-       C_INV };   // last corrected solve whose residual test failed
+       C_INV,     // last corrected solve whose residual test failed
+       C_DEL };   // last deletion whose rotations from the inverse failed their test
 
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }

@@ -1935,7 +1935,7 @@ struct Engine {
           I.rres[p0 + lane] = d;
           // |d| <= 2^-INV_BITS times the largest term (at least 2^(g - 2)); a
           // term that is not finite fails
-          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || I.guard_force) I.ctl[C_INV] = ep;
+          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || (I.guard_force && inner_step > 0)) I.ctl[C_INV] = ep;
         }
       }
       __syncthreads();
@@ -1955,6 +1955,77 @@ struct Engine {
     inv_product(np, I.rres, true);
     return sync();
   }
+  // Rotations of the downdate that deletes position q, from row q of the kept
+  // inverse (v, in the slot of the removed column).  v^T R~ = 0 for R without
+  // column q, and after rotations q .. t-1 the row they carry is v(q .. t)^T R~
+  // / h_t with h_t = |v(q .. t)|: rotation t has cos = v_{t+1} / h_{t+1}, sin =
+  // -h_t / h_{t+1}.  They come out of a prefix sum, all at once, where the
+  // chain over R itself (delete_position) takes 7 us per 32.  What they leave
+  // below the diagonal of column t is e_t = v(q .. t+1)^T R~_t / h_{t+1}, about
+  // eps |R~_t| as the inverse is kept by row operations (a small residual
+  // X R - I row by row); it is formed for every column, and where one is above
+  // 2^-47 |a_t| the chain takes the deletion and the inverse is given up.
+  static constexpr double DEL_TOL2 = 0x1p-94;
+  __device__ void inv_rotations(int q, int np, int nrot, int ep) {
+    double* sv = dyn;  // v(q .. np - 1)
+    __shared__ double sh[32];
+    const double* v = I.Rinv + (size_t)ldcg(I.rslot + np - 1) * I.ldr + q;
+    __syncthreads();
+    for (int j = tid; j <= nrot; j += NT) sv[j] = ldcg(v + j);
+    __syncthreads();
+    int lo, hi;
+    split(nrot, tm.size, tm.rank, lo, hi);  // nrot <= INV_ROWS: at most 32 each
+    if (lo < hi) {
+      double b = 0.0;
+      for (int j = tid; j <= lo; j += NT) b = fma(sv[j], sv[j], b);
+      b = block_sum(b, sh);  // h_lo^2
+      if (warp == 0) {
+        const int i = lo + lane;
+        const double vn = (i < hi) ? sv[i + 1] : 0.0;
+        double inc = vn * vn;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += t;
+        }
+        const double h2 = b + inc;
+        double hp = __shfl_up_sync(0xffffffffu, h2, 1);
+        if (lane == 0) hp = b;
+        if (i < hi) {
+          const double ih = rsqrt(h2);
+          I.rotc[i] = vn * ih;
+          I.rots[i] = -(i == 0 ? sv[0] : sqrt_gm(hp)) * ih;
+          if (!(h2 < 0x1p+1000) || !(b > 0x1p-900)) I.ctl[C_DEL] = ep;
+        }
+      }
+    }
+    // e_t of the column now at position q + i, a warp each
+    for (int i = tm.rank + tm.size * warp; i < nrot; i += tm.size * NW) {
+      const double* col = Rcol(ldcg(I.rslot + q + i)) + q;
+      const double an = ldcg(I.anorm + ldcg(I.order + q + i));
+      double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0;
+      for (int j0 = 0; j0 <= i + 1; j0 += 256) {
+        double r[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) r[u] = ldcg(col + min(j0 + 32 * u + lane, i + 1));
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          const int j = j0 + 32 * u + lane;
+          if (j <= i + 1) {
+            a0 = fma(r[u], sv[j], a0);
+            g0 = fma(sv[j], sv[j], g0);
+          }
+          if (j + 32 <= i + 1) {
+            a1 = fma(r[u + 1], sv[j + 32], a1);
+            g1 = fma(sv[j + 32], sv[j + 32], g1);
+          }
+        }
+      }
+      const double a = warp_sum(a0 + a1), g = warp_sum(g0 + g1);
+      if (lane == 0 && (!(a * a <= DEL_TOL2 * (an * an) * g) || I.guard_force)) I.ctl[C_DEL] = ep;
+    }
+  }
+
   // R y = rhs on [0, np) (the inner step's solve)
   __device__ bool solve_tri(int np) {
     if (!inv_on || np > INV_ROWS || (np <= INV_MIN && inv_n < np)) return trsv(np);
@@ -3327,6 +3398,27 @@ struct Engine {
     }
     if (!sync()) return false;
     phase(PH_CHAIN);
+    if (inv_n == np && nrot > 0) {
+      const int ep = ++iepoch;
+      inv_rotations(q, np, nrot, ep);
+      if (!sync()) return false;
+      if (ldcg(I.ctl + C_DEL) != ep) {
+        phase(PH_ZROT);
+        nP = np - 1;
+        rotate_columns(q, np, nrot, 0, false);
+        inv_n = np - 1;
+        const bool ok = sync();
+        phase(PH_INNER);
+        return ok;
+      }
+      inv_on = false;
+      inv_n = 0;
+      for (int i = tm.rank * NT + tid; i < nrot; i += tm.size * NT) {
+        I.rotc[i] = __longlong_as_double(0x7ff8000000000000LL);
+        I.rots[i] = __longlong_as_double(0x7ff8000000000000LL);
+      }
+      if (!sync()) return false;
+    }
     // (i) rotation chain: the rotations only (R's rotated rows are written
     // with the Z columns in (ii)).  Block b covers generating positions
     // [q + b*DB, q + (b+1)*DB) on CTA b mod size; lane l of warp 0 owns

@@ -55,14 +55,17 @@ def test_ill_conditioned(L, k_max, kappa):
 
 
 def test_given_up(L):
-    # the residual test forced to fail: substitution takes over
+    # the tests forced to fail in inner steps: with one column a block the
+    # inverse is there at the first deletion, whose rotations are tested (the
+    # chain takes over); with 24 an inner step makes it and tests the residual
+    # of its solve (substitution takes over)
     A, b, _ = WL.overdetermined_uniform(11, m=500, n=260)
     ctx = L.Context(500, 260)
     ctx.force_commit_guard(1)
-    for k_max in (1, 24):
+    for k_max, word in ((1, 12), (24, 11)):
         ref = O.nnls(A, b, k_max=k_max, trace=True)
         x, P, _, info = solve(L, ctx, A, b, k_max=k_max)
-        assert ctx.state("ctl", 16)[11] > 0  # a test failed, so the inverse was in use until then
+        assert ctx.state("ctl", 16)[word] > 0  # the test failed, so the inverse was in use until then
         assert_parity(x, P, info, ref, trace=ctx.trace())
     ctx.close()
 
