@@ -24,10 +24,11 @@ struct lhdm_ctx {
   int nsm = 0;
   int max_m = 0, max_n = 0, cap = 0, ldr = 0;
   ScratchLayout L{};
+  char* arena = nullptr;  // the one allocation that the pointers below share
   double* dscr = nullptr;
   int* iscr = nullptr;
   double* R = nullptr;
-  double* Rinv = nullptr;  // part of R's allocation; null: the solve substitutes
+  double* Rinv = nullptr;  // null: the solve substitutes
   int* rslot = nullptr;
   int* order = nullptr;
   double* xP = nullptr;
@@ -89,6 +90,12 @@ struct lhdm_batch {
 constexpr int MAX_DEVICES = 64;
 static std::mutex g_attr_mu;
 static std::atomic<bool> g_attr_done[MAX_DEVICES];
+
+// The barrier words and the error flag behind them (in one region) to zero
+// before a launch: one memset, not two.
+static cudaError_t clear_words(unsigned int* bar, int* err, cudaStream_t st) {
+  return cudaMemsetAsync(bar, 0, reinterpret_cast<char*>(err + 1) - reinterpret_cast<char*>(bar), st);
+}
 
 static int cuda_ok(cudaError_t e) { return e == cudaSuccess ? LHDM_OK : LHDM_ERR_CUDA; }
 
@@ -188,33 +195,51 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
   c->ldr = (c->cap + 1) & ~1;
   if ((max_n + c->nsm - 1) / c->nsm > CAND_LOCAL_MAX) { delete c; return LHDM_ERR_INVALID_ARG; }
   c->L = make_layout(max_m, max_n, c->nsm);
-  cudaError_t e = cudaSuccess;
-  e = cudaMalloc(&c->dscr, c->L.dtotal * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->iscr, c->L.itotal * sizeof(int));
-  // R and, behind it, its kept inverse (without it where memory is short)
-  const size_t nR = (size_t)c->ldr * c->cap;
-  if (e == cudaSuccess) {
-    if (cudaMalloc(&c->R, 2 * nR * sizeof(double)) == cudaSuccess) {
-      c->Rinv = c->R + nR;
-    } else {
-      cudaGetLastError();
-      e = cudaMalloc(&c->R, nR * sizeof(double));
-    }
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&c->rslot, (size_t)c->cap * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->order, (size_t)c->cap * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->xP, (size_t)c->cap * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->r, (size_t)std::max(max_m, 1) * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&c->nP, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->bar, 4 * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_info, sizeof(lhdm_info));
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_phase, (2 * NPHASE + 2) * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemset(c->d_phase, 0, (2 * NPHASE + 2) * sizeof(double));
+  // one allocation, carved in 256-byte granules: the words that start at zero
+  // first, R's kept inverse last (left out where memory is short); fourteen
+  // allocations cost a small context more than its solve
   c->trace_cap = 3 * max_n + 8;
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_trace, (size_t)6 * c->trace_cap * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_zero, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(c->d_zero, 0, sizeof(int));
+  const size_t nR = (size_t)c->ldr * c->cap;
+  size_t total = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return o;
+  };
+  const size_t o_phase = take((2 * NPHASE + 2) * sizeof(double)), o_zero = take(sizeof(int)), zeroed = total;
+  const size_t o_bar = take(4 * sizeof(unsigned int)), o_err = take(sizeof(int)), o_info = take(sizeof(lhdm_info)),
+               o_nP = take(sizeof(int)), o_rslot = take((size_t)c->cap * sizeof(int)),
+               o_order = take((size_t)c->cap * sizeof(int)), o_xP = take((size_t)c->cap * sizeof(double)),
+               o_r = take((size_t)std::max(max_m, 1) * sizeof(double)),
+               o_trace = take((size_t)6 * c->trace_cap * sizeof(int)), o_iscr = take(c->L.itotal * sizeof(int)),
+               o_dscr = take(c->L.dtotal * sizeof(double)), o_R = take(nR * sizeof(double)), without = total,
+               o_Rinv = take(nR * sizeof(double));
+  bool inv = true;
+  cudaError_t e = cudaMalloc(&c->arena, total);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    inv = false;
+    e = cudaMalloc(&c->arena, without);
+  }
+  if (e == cudaSuccess) {
+    char* p = c->arena;
+    c->d_phase = reinterpret_cast<double*>(p + o_phase);
+    c->d_zero = reinterpret_cast<int*>(p + o_zero);
+    c->bar = reinterpret_cast<unsigned int*>(p + o_bar);
+    c->err = reinterpret_cast<int*>(p + o_err);
+    c->d_info = reinterpret_cast<lhdm_info*>(p + o_info);
+    c->nP = reinterpret_cast<int*>(p + o_nP);
+    c->rslot = reinterpret_cast<int*>(p + o_rslot);
+    c->order = reinterpret_cast<int*>(p + o_order);
+    c->xP = reinterpret_cast<double*>(p + o_xP);
+    c->r = reinterpret_cast<double*>(p + o_r);
+    c->d_trace = reinterpret_cast<int*>(p + o_trace);
+    c->iscr = reinterpret_cast<int*>(p + o_iscr);
+    c->dscr = reinterpret_cast<double*>(p + o_dscr);
+    c->R = reinterpret_cast<double*>(p + o_R);
+    c->Rinv = inv ? reinterpret_cast<double*>(p + o_Rinv) : nullptr;
+    e = cudaMemset(p, 0, zeroed);
+  }
   if (e != cudaSuccess) {
     lhdm_destroy(c);
     return e == cudaErrorMemoryAllocation ? LHDM_ERR_ALLOC : LHDM_ERR_CUDA;
@@ -226,24 +251,11 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
 int lhdm_destroy(lhdm_ctx* c) {
   if (!c) return LHDM_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
-  cudaFree(c->dscr);
-  cudaFree(c->iscr);
-  cudaFree(c->R);
-  cudaFree(c->rslot);
-  cudaFree(c->order);
-  cudaFree(c->xP);
-  cudaFree(c->r);
-  cudaFree(c->nP);
-  cudaFree(c->bar);
-  cudaFree(c->err);
-  cudaFree(c->d_info);
-  cudaFree(c->d_phase);
-  cudaFree(c->d_trace);
+  cudaFree(c->arena);
   cudaFree(c->hA);
   cudaFree(c->hb);
   cudaFree(c->hx);
   cudaFree(c->hp);
-  cudaFree(c->d_zero);
   cudaFree(c->l1A);
   cudaFree(c->l1b);
   if (c->plan) lhdm_batch_destroy(c->plan);
@@ -294,8 +306,7 @@ int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, 
   I.bar_extra = c->stall_next ? 1 : 0;
   c->stall_next = false;
   c->have_state = false;
-  cudaError_t e = cudaMemsetAsync(c->bar, 0, 4 * sizeof(unsigned int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->err, 0, sizeof(int), st);
+  cudaError_t e = clear_words(c->bar, c->err, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   void* args[] = {(void*)&I, (void*)&c->bar, (void*)&c->err};
   e = cudaLaunchCooperativeKernel((const void*)lhdm_solve_grid_kernel, dim3(c->nsm), dim3(NT), args, DYN_SMEM, st);
@@ -440,8 +451,7 @@ int lhdm_backward(lhdm_ctx* c, int32_t idx, const double* A, int32_t lda, const 
   I.A = A;
   fill_ctx_inst(c, I);
   double* apu = c->dscr + c->L.apu;
-  cudaError_t e = cudaMemsetAsync(c->bar, 0, 4 * sizeof(unsigned int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->err, 0, sizeof(int), st);
+  cudaError_t e = clear_words(c->bar, c->err, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   double* apu_arg = dLdb ? dLdb : apu;
   void* args[] = {(void*)&I, (void*)&c->bar, (void*)&c->err, (void*)&dLdx, (void*)&dLdb,
@@ -639,8 +649,7 @@ extern "C" int lhdm_solve_noalloc(int32_t m, int32_t n, const double* A, int32_t
   cudaStream_t st = (cudaStream_t)stream;
   // the barrier words and the error flag must start at zero; everything
   // else is (re)initialised by the kernel itself
-  cudaError_t e = cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
+  cudaError_t e = clear_words(bar, err, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   void* args[] = {(void*)&I, (void*)&bar, (void*)&err};
   e = cudaLaunchCooperativeKernel((const void*)lhdm_solve_grid_kernel, dim3(d->nsm), dim3(NT), args, DYN_SMEM, st);
