@@ -1231,6 +1231,9 @@ struct Engine {
   __device__ bool trsv(int np) {
     if (np <= 0) return true;
     flops(cur_phase < 0 ? PH_SOLVE : cur_phase, (long long)np * np);
+    if constexpr (std::is_same<Team, CtaTeam>::value) {
+      if (np <= CTA_TRI) return trsv_cta(np);
+    }
     if (I.Dinv && tm.size >= 2 && np > 2 * TB) return trsv_pipelined(np);
     return trsv_blocked(np);
   }
@@ -1364,6 +1367,120 @@ struct Engine {
     return true;
   }
 
+
+  // One CTA: back substitution over 64-blocks from the last to the first.
+  // While warp 0 substitutes a block, the other warps stage the diagonal block
+  // before it (columns scaled by their reciprocal diagonal) and sum its rows
+  // over the columns solved already; then all warps add the block just solved.
+  // A block costs the substitution (64 steps of a shuffle, a load and an FMA)
+  // and about 3 000 cycles; with a barrier between all of this and its loads
+  // one after another it was 80 000 (500-row instances, R in HBM).
+  static constexpr int CTA_TRI = 4096;  // y in shared memory
+  __device__ bool trsv_cta(int np) {
+    const int nb = (np + TB - 1) / TB;
+    constexpr int DS = TB + 1;
+    double* sD0 = dyn;                  // two diagonal blocks, column c at c DS
+    double* sRi = sD0 + 2 * TB * DS;    // their reciprocal diagonals
+    double* sA = sRi + 2 * TB;          // NW x TB partial sums
+    double* sy = sA + NW * TB;          // np
+    int* ss = reinterpret_cast<int*>(sy + np);  // slots
+    auto stage = [&](int bi, int w, int nw) {
+      const int b0 = bi * TB, nbk = min(np, b0 + TB) - b0;
+      double* sD = sD0 + (bi & 1) * TB * DS;
+      double* ri = sRi + (bi & 1) * TB;
+      for (int c0 = w; c0 < nbk; c0 += 4 * nw) {
+        double v0[4], v1[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int c = min(c0 + k * nw, nbk - 1);
+          const double* col = Rcol(ss[b0 + c]) + b0;
+          v0[k] = ldcg(col + min(lane, c));
+          v1[k] = ldcg(col + min(lane + 32, c));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int c = c0 + k * nw;
+          if (c >= nbk) break;
+          const double d = __shfl_sync(0xffffffffu, c < 32 ? v0[k] : v1[k], c & 31);
+          const double r = rcp_nr(d);
+          if (lane < c) sD[c * DS + lane] = v0[k] * r;
+          if (lane + 32 < c) sD[c * DS + lane + 32] = v1[k] * r;
+          if (lane == 0) ri[c] = r;
+        }
+      }
+    };
+    __syncthreads();
+    for (int c = tid; c < np; c += NT) ss[c] = ldcg(I.rslot + c);
+    __syncthreads();
+    stage(nb - 1, warp, NW);
+    double p0 = 0.0, p1 = 0.0;  // this warp's sums for rows lane, lane + 32 of the coming block
+    // columns c0 + w, c0 + w + nw, .. < c1 on the rows of block bi
+    auto add = [&](int bi, int c0, int c1, int w, int nw) {
+      const int r = bi * TB + lane;
+      for (int c = c0 + w; c < c1; c += 8 * nw) {
+        double v0[8], v1[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const double* col = Rcol(ss[min(c + k * nw, c1 - 1)]) + r;
+          v0[k] = ldcg(col);
+          v1[k] = ldcg(col + 32);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (c + k * nw < c1) {
+            const double y = sy[c + k * nw];
+            p0 = fma(v0[k], y, p0);
+            p1 = fma(v1[k], y, p1);
+          }
+      }
+    };
+    for (int bi = nb - 1; bi >= 0; --bi) {
+      const int b0 = bi * TB, b1 = min(np, b0 + TB), nbk = b1 - b0;
+      sA[warp * TB + lane] = p0;
+      sA[warp * TB + lane + 32] = p1;
+      p0 = p1 = 0.0;
+      __syncthreads();
+      if (warp == 0) {
+        const double* sD = sD0 + (bi & 1) * TB * DS;
+        const double* ri = sRi + (bi & 1) * TB;
+        double a0 = (lane < nbk) ? ldcg(I.rhs + b0 + lane) : 0.0, a1 = (lane + 32 < nbk) ? ldcg(I.rhs + b0 + lane + 32) : 0.0;
+        if (bi + 1 < nb) {
+          double t0[4] = {0.0, 0.0, 0.0, 0.0}, t1[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            t0[w & 3] += sA[w * TB + lane];
+            t1[w & 3] += sA[w * TB + lane + 32];
+          }
+          a0 -= (t0[0] + t0[1]) + (t0[2] + t0[3]);
+          a1 -= (t1[0] + t1[1]) + (t1[2] + t1[3]);
+        }
+        // a_i -= (R_ij / R_jj) a_j, j from the last row up; y_j = a_j / R_jj
+        for (int j = nbk - 1; j >= 32; --j) {
+          const double aj = __shfl_sync(0xffffffffu, a1, j & 31);
+          a0 = fma(-sD[j * DS + lane], aj, a0);
+          if (lane + 32 < j) a1 = fma(-sD[j * DS + lane + 32], aj, a1);
+        }
+        for (int j = min(nbk, 32) - 1; j >= 0; --j) {
+          const double aj = __shfl_sync(0xffffffffu, a0, j);
+          if (lane < j) a0 = fma(-sD[j * DS + lane], aj, a0);
+        }
+        if (lane < nbk) {
+          sy[b0 + lane] = a0 * ri[lane];
+          I.yP[b0 + lane] = sy[b0 + lane];
+        }
+        if (lane + 32 < nbk) {
+          sy[b0 + lane + 32] = a1 * ri[lane + 32];
+          I.yP[b0 + lane + 32] = sy[b0 + lane + 32];
+        }
+      } else if (bi > 0) {
+        stage(bi - 1, warp - 1, NW - 1);
+        add(bi - 1, b1, np, warp - 1, NW - 1);
+      }
+      __syncthreads();
+      if (bi > 0) add(bi - 1, b0, b1, warp, NW);
+    }
+    return sync();
+  }
 
   // Flag-pipelined back substitution (teams of several CTAs).  Positions are
   // cut into TB-blocks; rank 0 walks them from the last to the first and is
@@ -3944,11 +4061,18 @@ struct Engine {
         const int hl = lane >> 4, il = lane & 15;
         for (int t0 = 0; t0 < gmax; t0 += TR) {
           // rows q+t0+1 .. q+t0+TR (the bots of rotations t0 ..)
-          for (int cc = 0; cc < 32; cc += 2) {
-            const int c = cc + hl;
-            const double* cp = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<long long>(colp), c));
-            const int ns_c = __shfl_sync(0xffffffffu, nsu, c);
-            sT[il * 33 + c] = (t0 + il < ns_c) ? ldcg(cp + q + t0 + 1 + il) : 0.0;
+          // (eight loads in flight; a column without these rows reads its first)
+          for (int cc = 0; cc < 32; cc += 16) {
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int c = cc + 2 * k + hl;
+              const double* cp = reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, reinterpret_cast<long long>(colp), c));
+              const int ns_c = __shfl_sync(0xffffffffu, nsu, c);
+              v[k] = ldcg(cp + (t0 + il < ns_c ? q + t0 + 1 + il : 0));
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sT[il * 33 + cc + 2 * k + hl] = v[k];
           }
           __syncwarp();
 #pragma unroll 4
@@ -4249,21 +4373,41 @@ struct Engine {
           const int i1 = (k == kl) ? (int)(e1 - (long long)k * m) : m;
           const double* a = I.A + (size_t)s_zl[k] * I.lda;
           double s0 = 0.0, s1 = 0.0;
-          int i = i0 + lane;
-          for (; i + 224 < i1; i += 256) {
-            double av[8], rr[8];
+          if constexpr (std::is_same<Team, CtaTeam>::value) {
+            // sixteen loads in flight, the last rows' included (clamped, against
+            // zeros of r; A is finite): A comes from HBM here, and one load at a
+            // time for the last rows took longer than the rest of a 500-row
+            // column (760 -> 400 kcycles at 506 x 1012)
+            for (int b0 = i0; b0 < i1; b0 += 512) {
+              double av[16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              av[j] = __ldg(a + i + 32 * j);
-              rr[j] = r_in_smem ? rv[i + 32 * j] : ldcg(rv + i + 32 * j);
-            }
+              for (int j = 0; j < 16; ++j) av[j] = __ldg(a + min(b0 + lane + 32 * j, i1 - 1));
 #pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-              s0 = fma(av[j], rr[j], s0);
-              s1 = fma(av[j + 1], rr[j + 1], s1);
+              for (int j = 0; j < 16; ++j) {
+                if (b0 + 32 * j >= i1) break;
+                const int i = b0 + lane + 32 * j;
+                const double rr = i < i1 ? (r_in_smem ? rv[i] : ldcg(rv + i)) : 0.0;
+                if (j & 1) s1 = fma(av[j], rr, s1);
+                else s0 = fma(av[j], rr, s0);
+              }
             }
+          } else {
+            int i = i0 + lane;
+            for (; i + 224 < i1; i += 256) {
+              double av[8], rr[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                av[j] = __ldg(a + i + 32 * j);
+                rr[j] = r_in_smem ? rv[i + 32 * j] : ldcg(rv + i + 32 * j);
+              }
+#pragma unroll
+              for (int j = 0; j < 8; j += 2) {
+                s0 = fma(av[j], rr[j], s0);
+                s1 = fma(av[j + 1], rr[j + 1], s1);
+              }
+            }
+            for (; i < i1; i += 32) s0 = fma(__ldg(a + i), r_in_smem ? rv[i] : ldcg(rv + i), s0);
           }
-          for (; i < i1; i += 32) s0 = fma(__ldg(a + i), r_in_smem ? rv[i] : ldcg(rv + i), s0);
           const double tot = warp_sum(s0 + s1);
           if (lane == 0) {
             if (k == kf) s_pp[warp][0] = tot;
