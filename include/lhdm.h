@@ -306,9 +306,12 @@ int lhdm_set_wait_limit(lhdm_ctx* ctx, int64_t ns);
  * products on bf16 tensor cores, with a fallback to FP64 where the digits
  * could be less accurate than an FP64 evaluation): mode 1 sends every batch
  * of the later solves on ctx to the FP64 path as the guard would, mode 0
- * restores the guard's own decisions.  Results must not change beyond
- * rounding; the count of batches sent is word [10] of the "ctl" state of
- * lhdm_debug_state.  Errors: INVALID_ARG.
+ * restores the guard's own decisions.  Mode 1 also fails the tests of the
+ * kept inverse of R in inner steps, so that substitution and the rotation
+ * chain take over.  Results must not change beyond rounding; the count of
+ * batches sent is word [10] of the "ctl" state of lhdm_debug_state, [11] and
+ * [12] are nonzero after a failed test of a solve and of a deletion.
+ * Errors: INVALID_ARG.
  */
 int lhdm_debug_commit_guard(lhdm_ctx* ctx, int32_t mode);
 
@@ -350,16 +353,18 @@ int lhdm_trace(lhdm_ctx* ctx, int32_t* out, int32_t max_rows, void* stream);
  * "W" (ld = max_m rounded up to even), "R" (slot-major, ld = the context's
  * min(max_m, max_n) rounded up to even), "ctl" (16 int32 control words;
  * [10] = commit batches that the accuracy guard of the tensor-core commit
- * sent to FP64).  FP64 except the int32 arrays.  Errors: INVALID_ARG for an unknown name or count too large. */
+ * sent to FP64, [11] and [12] nonzero after a failed test of the kept
+ * inverse).  FP64 except the int32 arrays.  Errors: INVALID_ARG for an unknown name or count too large. */
 int lhdm_debug_state(lhdm_ctx* ctx, const char* name, void* host, int64_t count, void* stream);
 
 /* Profile of the last solve on ctx.  ms[0..12) = device time in ms of each
  * solver phase: setup, DM, panel, triangular solve (outer step), commit,
  * inner-loop control and bookkeeping, residual, dual vector, feasibility
- * loop, Givens chain on R, rotations of the Z columns, triangular solves of
- * the inner loop; ms[12..24) = the algorithmic FP64 flops of the same
+ * loop, the downdates' rotations (with their application where the Givens
+ * chain generates them), their application, triangular solves of the inner
+ * loop; ms[12..24) = the algorithmic FP64 flops of the same
  * phases (an FMA counts 2); ms[24] = bf16 tensor-core MMA instructions
- * (m16n8k16, 4096 flops each) the commit issued.  Writes min(n, 25) values
+ * (tcgen05, in units of m16n8k16 = 4096 flops) the commit issued.  Writes min(n, 25) values
  * and returns how many (negative status on error).  Synchronises the
  * stream. */
 int lhdm_phase_times(lhdm_ctx* ctx, double* ms, int32_t n, void* stream);
