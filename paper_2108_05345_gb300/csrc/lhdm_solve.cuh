@@ -1561,6 +1561,10 @@ struct Engine {
       cp_commit();
       if (g == 0 && row < nbk && bi + 2 < nb) pacc = ldcg(I.accb + b0 + row);
     };
+    // the last block may be short: its missing y meet the zero columns of sRT
+    // in the block before it, and what shared memory holds at launch may be NaN
+    if (tid < 2 * TB) s_y[tid / TB][tid & (TB - 1)] = 0.0;
+    __syncthreads();
     prefetch(nb - 1);
     for (int bi = nb - 1; bi >= 0; --bi) {
       const int b0 = bi * TB, nbk = min(np, b0 + TB) - b0;
