@@ -291,12 +291,6 @@ __device__ __forceinline__ unsigned dig2(unsigned wa, unsigned wb, int sh, unsig
   const unsigned p = ((wa >> sh) & 0x7Fu) | (((wb >> sh) & 0x7Fu) << 16) | 0x43004300u;
   return bf16x2_fma(p, sg, nb);
 }
-// a bf16 pair times 2^-7 (exact for the 7-bit digits: no bits are lost)
-__device__ __forceinline__ unsigned bf16x2_scale_m7(unsigned x) {
-  unsigned r;
-  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(0x3C003C00u), "r"(0x80008000u));
-  return r;
-}
 // digit k (0..7) of a value given as 28-bit halves
 __device__ __forceinline__ unsigned dig2k(int k, unsigned ha, unsigned la, unsigned hb, unsigned lb, unsigned sg,
                                           unsigned nb) {
@@ -305,11 +299,6 @@ __device__ __forceinline__ unsigned dig2k(int k, unsigned ha, unsigned la, unsig
 }
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void ldsm_x4(unsigned* r, const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(smem_u32(p)));
-}
 __device__ __forceinline__ void ldsm_x4_t(unsigned* r, const void* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -326,21 +315,11 @@ __device__ __forceinline__ void mma_bf16(float* c, const unsigned* a, const unsi
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// 16-byte asynchronous copy global -> shared (zero fill when !ok)
-__device__ __forceinline__ void cp16(void* dst, const void* src, bool ok) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)
-               : "memory");
-}
 // 8- and 4-byte asynchronous copies global -> shared (zero fill when !ok)
 __device__ __forceinline__ void cp8(void* dst, const void* src, bool ok) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 8 : 0)
                : "memory");
 }
-__device__ __forceinline__ void cp4(void* dst, const void* src, bool ok) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 4 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // mbarrier and bulk (TMA) copies global -> shared
