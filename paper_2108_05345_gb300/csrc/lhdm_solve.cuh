@@ -690,6 +690,7 @@ struct Engine {
           vd_store_row(rr, va, v0a, vb, v0b);
         }
         vd_store_tail(L);
+        publish_digits();
         vd_ok = true;
       }
     }
@@ -734,6 +735,14 @@ struct Engine {
   __device__ __forceinline__ void vd_store_tail(int L) {
     const int end = ((((nP + L - 1) >> 3) + 2) << 3) - nP;
     for (int r = L + warp; r < end; r += NW) vd_store_row(r, 0.0, 1.0, 0.0, 1.0);
+  }
+  // Every thread after its digit stores, before the barrier that ends the
+  // panel: the commit reads Vd with bulk copies, which go through the async
+  // proxy and past L1, and a barrier alone orders ordinary accesses only.  The
+  // one-CTA barrier is no fence beyond the CTA, so that team adds one.
+  __device__ __forceinline__ void publish_digits() {
+    if constexpr (std::is_same<Team, CtaTeam>::value) __threadfence();
+    fence_proxy_async_all();
   }
 
   // Panel with the team's rows held in shared memory (at most PR_MAX rows
@@ -1115,6 +1124,7 @@ struct Engine {
                      (t2 < kk) ? (row > t2 ? sP[rr * PS + t2] : (row == t2 ? v0b : 0.0)) : 0.0, v0b);
       }
       if (tm.rank == P - 1) vd_store_tail(L);
+      publish_digits();
     }
     if (tm.rank == 0) {
       // T is the inverse of the upper triangle M with M[r][r] = 1/beta_r and
@@ -2630,7 +2640,10 @@ struct Engine {
       s_Ec[tid] = -8000;
       s_cp[tid] = commit_col(cs.s_cid, tid < nb ? tid : 0) + r0d;
     }
-    fence_proxy_async();  // generic writes of the work area before the async copies into it
+    // ordinary writes before the async copies: the panel's digits (published
+    // by their writers, acquired by the barrier that ended the panel) and the
+    // work area
+    fence_proxy_async_all();
     __syncthreads();
     // column scales of C' = 2^Er C: a warp takes every NW-th group of 128
     // rows of all columns, sixteen loads in flight (clamped, not predicated:
