@@ -95,7 +95,7 @@ inline ScratchLayout make_layout(int max_m, int max_n, int team) {
   L.ctl = take(16);
   L.qlist = take(cap);
   L.tflag = take(L.pipelined ? nbk * (1 + TB / SLAB + INV_PARTS) : 1);
-  L.Ver = take(m + 32);
+  L.Ver = take(m + 64);  // pass 1 of the commit reads whole chunks of up to 64 rows
   L.csign = take(n);
   L.itotal = o;
   return L;

@@ -2760,8 +2760,9 @@ struct Engine {
         const double* col = s_cp[c];
         const int dec = (live && s_Ec[c] > -8000) ? s_Ec[c] + 1022 : 1 << 20;
         // rows 16 p + 2 drp + {0, 1, 8, 9} of unit g (chunk g / upc, p = g %
-        // upc); rows past the last one read what follows in the scratch
-        // region and count as zero
+        // upc); rows past the last one, at most 63, count as zero: Ver has
+        // room for them, a column reads into the next one, into Q^T b or into
+        // the vectors behind it
         double2 xa, xb;
         int2 ea, eb;
         auto load_u = [&](int g) {
