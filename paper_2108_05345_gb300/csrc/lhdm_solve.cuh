@@ -2004,6 +2004,7 @@ struct Engine {
         if (lane + 32 < k) row[c0 + lane + 32] = a1 * sri[lane + 32];
       }
     }
+    __syncthreads();  // the first append goes on to the commit, which overwrites dyn, without a team barrier
   }
 
   // Residual rhs - R yP on rows [0, np) into rres, eight rows per CTA and
