@@ -316,6 +316,18 @@ int lhdm_set_wait_limit(lhdm_ctx* ctx, int64_t ns);
 int lhdm_debug_commit_guard(lhdm_ctx* ctx, int32_t mode);
 
 /*
+ * Failure-detection test aids: what goes wrong in the later lhdm_solve calls
+ * on ctx, as a sum of the bits below (0: nothing, the state of a new context).
+ * LHDM_INJECT_COMMIT_STALL: the tensor-core commit leaves out the last
+ * arrivals its matrix products wait for; every wait of the commit runs out
+ * (4 s), what was in flight is waited for, and the solve returns
+ * LHDM_ERR_TIMEOUT; the context stays usable.  Errors: INVALID_ARG.
+ */
+#define LHDM_INJECT_COMMIT_STALL 1
+#define LHDM_INJECT_ALL 1
+int lhdm_debug_inject(lhdm_ctx* ctx, int32_t what);
+
+/*
  * Failure-detection test aid: the next lhdm_solve on ctx runs with a grid
  * barrier that expects one arrival more than the grid has, so no CTA ever
  * releases it, every CTA's bounded wait runs out (lhdm_set_wait_limit) and

@@ -52,6 +52,7 @@ struct lhdm_ctx {
   long long wait_ns = 0;
   bool stall_next = false;
   int guard_force = 0;  // test aid for the tensor-core commit's accuracy guard
+  int inject = 0;       // test aid: LHDM_INJECT_* bits of later solves
   // batched solves: the plan of the last lhdm_solve_batched and the
   // arguments it was made for (reused while they repeat)
   int max_batch = 0;
@@ -279,6 +280,7 @@ static void fill_ctx_inst(lhdm_ctx* c, Inst& I) {
   I.trace_cap = c->trace_cap;
   I.wait_ns = c->wait_ns > 0 ? c->wait_ns : WAIT_NS;
   I.guard_force = c->guard_force;
+  I.inject = c->inject;
 }
 
 int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, const double* b,
@@ -515,6 +517,12 @@ int lhdm_set_wait_limit(lhdm_ctx* c, int64_t ns) {
 int lhdm_debug_commit_guard(lhdm_ctx* c, int32_t mode) {
   if (!c || mode < 0 || mode > 1) return LHDM_ERR_INVALID_ARG;
   c->guard_force = mode;
+  return LHDM_OK;
+}
+
+int lhdm_debug_inject(lhdm_ctx* c, int32_t what) {
+  if (!c || (what & ~LHDM_INJECT_ALL)) return LHDM_ERR_INVALID_ARG;
+  c->inject = what;
   return LHDM_OK;
 }
 

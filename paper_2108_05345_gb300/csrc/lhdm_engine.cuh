@@ -136,7 +136,8 @@ struct Inst {
                               // expects beyond the grid (0 in every normal solve)
   int guard_force;            // test aid: 1 sends every tensor-core commit batch to
                               // FP64 as the accuracy guard would, and fails the tests
-                          // of the kept inverse in inner steps (0 in normal solves)
+                              // of the kept inverse in inner steps (0 in normal solves)
+  int inject;                 // test aid: LHDM_INJECT_* bits (0 in normal solves)
   DevParams prm;
 };
 

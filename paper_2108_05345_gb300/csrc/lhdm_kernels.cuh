@@ -142,6 +142,7 @@ inline __host__ __device__ void bind_scratch(Inst& I, const ScratchLayout& L, do
   I.wait_ns = WAIT_NS;
   I.bar_extra = 0;
   I.guard_force = 0;
+  I.inject = 0;
 }
 
 // CTA barriers and tensor memory of the tensor-core commit (every thread of
@@ -150,16 +151,17 @@ struct TcState {
   unsigned long long* mbs;
   unsigned tmem;
 };
+constexpr int TC_BARS = 18;
 inline __device__ void tc_barriers(unsigned long long* mb) {
   if (threadIdx.x == 0) {
-    // V tiles and MMA completions: one arrival; pass-1 slots: C digits worth
-    // 8 and V's copy; accumulator reads: one per warp
-    for (int i = 0; i < 17; ++i) mbar_init(mb + i, i < 5 ? 1 : i < 10 ? 9 : i < 15 ? 1 : NW);
+    // V's copies and MMA completions: one arrival; pass-1 slots: C digits
+    // worth 8; accumulator reads and a failed commit's MMAs: one per warp
+    for (int i = 0; i < TC_BARS; ++i) mbar_init(mb + i, i < 5 ? 1 : i < 10 ? 8 : i < 15 ? 1 : NW);
     fence_mbar_init();
   }
 }
 inline __device__ TcState tc_open() {
-  __shared__ unsigned long long s_mb[17];
+  __shared__ unsigned long long s_mb[TC_BARS];
   __shared__ unsigned s_tmem;
   if (threadIdx.x < 32) tmem_alloc(&s_tmem);
   tc_barriers(s_mb);
@@ -168,11 +170,12 @@ inline __device__ TcState tc_open() {
   tc_fence_after();
   return TcState{s_mb, s_tmem};
 }
-// after a wait ran out: fresh barriers for the CTA's next instance
+// after a wait ran out (and the commit has drained what was in flight):
+// fresh barriers for the CTA's next instance
 inline __device__ void tc_reset(const TcState& t) {
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int i = 0; i < 17; ++i) mbar_inval(t.mbs + i);
+    for (int i = 0; i < TC_BARS; ++i) mbar_inval(t.mbs + i);
   tc_barriers(t.mbs);
   __syncthreads();
 }

@@ -2067,7 +2067,7 @@ struct Engine {
           I.rres[p0 + lane] = d;
           // |d| <= 2^-INV_BITS times the largest term (at least 2^(g - 2)); a
           // term that is not finite fails
-          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || (I.guard_force && inner_step > 0)) I.ctl[C_INV] = ep;
+          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || (I.guard_force == 1 && inner_step > 0)) I.ctl[C_INV] = ep;
         }
       }
       __syncthreads();
@@ -2154,7 +2154,7 @@ struct Engine {
         }
       }
       const double a = warp_sum(a0 + a1), g = warp_sum(g0 + g1);
-      if (lane == 0 && (!(a * a <= DEL_TOL2 * (an * an) * g) || I.guard_force)) I.ctl[C_DEL] = ep;
+      if (lane == 0 && (!(a * a <= DEL_TOL2 * (an * an) * g) || I.guard_force == 1)) I.ctl[C_DEL] = ep;
     }
   }
 
@@ -2524,13 +2524,17 @@ struct Engine {
   static constexpr float GUARD1 = 2048.0f;  // 2^11: sum |v'||c'| >= 2^(Ec-3)
   static constexpr unsigned ABS2 = 0x7FFF7FFFu;  // clears the signs of a bf16 pair
 
-  // CTA barriers of the tensor-core commit (mbs): V tiles arrived (bulk
-  // copies), a pass-1 slot's V chunk arrived and its C digits written
-  // (arrivals worth 8 per chunk and the copy's), MMAs of a slot complete,
-  // accumulators of a pass-2 half read (one arrival per warp).  mpar holds the parity of each barrier's current phase.
-  enum { MB_V = 0, MB_C = 5, MB_F = 10, MB_T = 15 };
+  // CTA barriers of the tensor-core commit (mbs): a pass-1 slot's V chunk or
+  // a pass-2 V tile arrived (bulk copy), a slot's C digits written (arrivals
+  // worth 8 per chunk), MMAs of a slot complete, accumulators of a pass-2
+  // half read (one arrival per warp), and what a failed commit leaves in
+  // flight (one arrival per warp).  mpar holds the parity of each barrier's
+  // current phase.
+  enum { MB_V = 0, MB_C = 5, MB_F = 10, MB_T = 15, MB_D = 17 };
   // Bounded wait for the phase `ahead` uses after the current one of barrier
-  // i; a thread whose wait ran out does not wait again.
+  // i; a thread whose wait ran out does not wait again.  Its warp leaves the
+  // pass: an arrival on a barrier whose phase has not completed would count
+  // for that phase.
   __device__ __forceinline__ void mb_wait(int i, int ahead, bool& ok) {
     if (!ok) return;
     const unsigned par = ((mpar >> i) ^ (unsigned)ahead) & 1u;
@@ -2543,6 +2547,22 @@ struct Engine {
         return;
       }
     }
+  }
+  // After a wait ran out (every thread): waits, again with a limit, for the
+  // MMAs the warps issued and for the bulk copies, staged[i] of them on
+  // barrier MB_V + i in this pass, so that nothing writes the CTA's shared
+  // memory or tensor memory after it leaves the commit.
+  __device__ void drain_tc(const unsigned* staged) {
+    if (mma_thread(warp)) umma_commit(mbs + MB_D);
+    __syncwarp();
+    bool ok = true;
+    mb_wait(MB_D, 0, ok);
+    for (int i = 0; i < MB_C; ++i)
+      if (staged[i] > 0u) {
+        ok = true;
+        mb_wait(MB_V + i, (int)staged[i] - 1, ok);
+      }
+    __syncthreads();
   }
 
   // Digits l the M tile mt of pass 1 takes (MT = KP / 16 tiles of 128 pairs
@@ -2582,6 +2602,7 @@ struct Engine {
     constexpr int G1 = p1_groups(MT), NR = p1_slots(MT);
     constexpr unsigned VB = G1 * MT * 2048, CBB = G1 * ND * (NB / 8) * 128;
     for (int j = 0; j < n; ++j) {
+      mb_wait(MB_V + slot, use, ok);
       mb_wait(MB_C + slot, use, ok);
       if (!ok) return;
       tc_fence_after();
@@ -2630,13 +2651,16 @@ struct Engine {
     const int* ver = I.Ver + r0d + (nP & 7);  // 32-byte aligned, like the columns' rows (16)
     __shared__ int s_Ec[CB], s_Ee[CB];
     __shared__ double* s_cp[CB];  // columns from the first digit row on (absent ones: the first)
+    __shared__ unsigned s_stg[MB_C];  // bulk copies of the pass per barrier
     bool ok = true;
     auto expired = [&]() {
       if (tid == 0) {
         int* er = tm_err();
         if (er) atomicExch(er, 1);
       }
+      drain_tc(s_stg);
     };
+    if (tid < MB_C) s_stg[tid] = 0u;
     if (tid < CB) {
       s_Ec[tid] = -8000;
       s_cp[tid] = commit_col(cs.s_cid, tid < nb ? tid : 0) + r0d;
@@ -2744,8 +2768,9 @@ struct Engine {
             if (j >= NR) mb_wait(MB_F + slot, use - 1, ok);
             if (!ok) break;
             const unsigned bytes = (unsigned)groups(j) * RGB;
-            mbar_expect_tx(mbs + MB_C + slot, bytes);
-            bulk_g2s(sV + slot * G1 * RGB, gV + (size_t)chunk(j) * G1 * RGB, bytes, mbs + MB_C + slot);
+            s_stg[slot] = (unsigned)use + 1u;
+            mbar_expect_tx(mbs + MB_V + slot, bytes);
+            bulk_g2s(sV + slot * G1 * RGB, gV + (size_t)chunk(j) * G1 * RGB, bytes, mbs + MB_V + slot);
             if (++slot == NR) { slot = 0; ++use; }
           }
         }
@@ -2800,6 +2825,10 @@ struct Engine {
           }
           if (g + nw < ug) load_u(g + nw);
           if (j >= NR) mb_wait(MB_F + s, u - 1, ok);
+          if (!__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            break;
+          }
           unsigned char* pp = sC + s * CBB + (p * 2 * ND * NG + cg) * 128 + (lane & 7) * 16 + drp * 4;
 #pragma unroll
           for (int q = 0; q < 4; q += 2) {
@@ -2816,7 +2845,7 @@ struct Engine {
           }
           fence_proxy_async();  // the digits before the MMAs read them
           __syncwarp();
-          if (lane == 0) mbar_arrive(mbs + MB_C + s, 8 >> (ush + NG - 1));
+          if (lane == 0 && !((I.inject & LHDM_INJECT_COMMIT_STALL) && j == nch - 1)) mbar_arrive(mbs + MB_C + s, 8 >> (ush + NG - 1));
           s += ((g + nw) >> ush) - (g >> ush);  // at most NR on
           if (s >= NR) { s -= NR; ++u; }
         }
@@ -2832,7 +2861,7 @@ struct Engine {
       __syncthreads();
     }
     for (int s = 0; s < NR; ++s)
-      if (((nch - s + NR - 1) / NR) & 1) mpar ^= 0x420u << s;  // uses of slot s
+      if (((nch - s + NR - 1) / NR) & 1) mpar ^= 0x421u << s;  // uses of slot s
     // Guard, first on the chunks still in shared memory (the last NR): sums
     // of |leading digit| products per (reflector, column), a warp's 16
     // reflectors x 8 columns x 16 rows; any rows' sum is a lower bound.
@@ -3012,9 +3041,11 @@ struct Engine {
     auto stage_t = [&](int i) {  // one thread
       const int b = dbl ? i & 1 : 0;
       const unsigned bytes = (unsigned)min(16, ngr - tile(i) * 16) * RGB;
+      s_stg[b] += 1u;
       mbar_expect_tx(mbs + MB_V + b, bytes);
       bulk_g2s(sW + b * 16 * RGB, gV + (size_t)tile(i) * 16 * RGB, bytes, mbs + MB_V + b);
     };
+    if (tid < MB_C) s_stg[tid] = 0u;
     fence_proxy_async();  // the work area's generic accesses before the async copies
     __syncthreads();
     if (tid == 0) {
@@ -3097,7 +3128,11 @@ struct Engine {
     for (int i = 0; i < nt2; ++i) {
       if (dbl && i + 1 < nt2) issue2(i + 1);
       mb_wait(MB_F + (i & 1), i >> 1, ok);
-      if (tid == 32 * (i & (NW - 1)) && ok) {  // tile i's V buffer is free
+      if (!__all_sync(0xffffffffu, ok)) {
+        ok = false;
+        break;
+      }
+      if (tid == 32 * (i & (NW - 1))) {  // tile i's V buffer is free
         const int nx = i + (dbl ? 2 : 1);
         if (nx < nt2) stage_t(nx);
       }

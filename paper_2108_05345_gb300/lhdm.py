@@ -24,6 +24,7 @@ LHDM_ERR_TIMEOUT = 6
 LHDM_ERR_ALLOC = 7
 LHDM_ERR_NO_STATE = 8
 LHDM_ERR_TOO_LARGE = 9
+LHDM_INJECT_COMMIT_STALL = 1
 KMAX_LIMIT = 64
 MODE_NNLS, MODE_SIGNED, MODE_SIGNED_FLIP = 0, 1, 2
 PHASES = ("setup", "dm", "panel", "solve", "commit", "inner", "residual", "dual",
@@ -77,6 +78,7 @@ def lib():
         L.lhdm_solve_l1.argtypes = [V, i32, i32, d, i32, d, C.c_double, P, d, d, I, V]
         L.lhdm_debug_stall_next_solve.argtypes = [V]
         L.lhdm_debug_commit_guard.argtypes = [V, i32]
+        L.lhdm_debug_inject.argtypes = [V, i32]
         L.lhdm_debug_fast_math.argtypes = [V, V, i32, V]
         L.lhdm_phase_times.argtypes = [V, C.POINTER(C.c_double), i32, V]
         L.lhdm_trace.argtypes = [V, C.POINTER(C.c_int32), i32, V]
@@ -348,6 +350,10 @@ class Context:
 
     def force_commit_guard(self, mode):
         _check(lib().lhdm_debug_commit_guard(self.h, int(mode)), "lhdm_debug_commit_guard")
+
+    def inject(self, what):
+        """Failure-detection test aid (lhdm_debug_inject)."""
+        _check(lib().lhdm_debug_inject(self.h, int(what)), "lhdm_debug_inject")
 
     def stall_next_solve(self):
         _check(lib().lhdm_debug_stall_next_solve(self.h), "lhdm_debug_stall_next_solve")
