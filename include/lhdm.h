@@ -328,6 +328,14 @@ int lhdm_debug_commit_guard(lhdm_ctx* ctx, int32_t mode);
 int lhdm_debug_inject(lhdm_ctx* ctx, int32_t what);
 
 /*
+ * Test aid for GPUs (or slices of one) with fewer SMs: the later lhdm_solve
+ * calls on ctx run on `ctas` CTAs, 2 up to the SM count (0: one per SM, the
+ * state of a new context).  Errors: INVALID_ARG, also when a CTA's share of
+ * the context's columns would not fit.
+ */
+int lhdm_debug_set_ctas(lhdm_ctx* ctx, int32_t ctas);
+
+/*
  * Failure-detection test aid: the next lhdm_solve on ctx runs with a grid
  * barrier that expects one arrival more than the grid has, so no CTA ever
  * releases it, every CTA's bounded wait runs out (lhdm_set_wait_limit) and

@@ -53,6 +53,7 @@ struct lhdm_ctx {
   bool stall_next = false;
   int guard_force = 0;  // test aid for the tensor-core commit's accuracy guard
   int inject = 0;       // test aid: LHDM_INJECT_* bits of later solves
+  int ctas = 0;         // CTAs of a solve: the SM count (test aid: fewer)
   // batched solves: the plan of the last lhdm_solve_batched and the
   // arguments it was made for (reused while they repeat)
   int max_batch = 0;
@@ -192,6 +193,7 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
   c->max_m = max_m;
   c->max_n = max_n;
   c->max_batch = max_batch;
+  c->ctas = c->nsm;
   c->cap = std::max(std::min(max_m, max_n), 1);
   c->ldr = (c->cap + 1) & ~1;
   if ((max_n + c->nsm - 1) / c->nsm > CAND_LOCAL_MAX) { delete c; return LHDM_ERR_INVALID_ARG; }
@@ -311,7 +313,7 @@ int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, 
   cudaError_t e = clear_words(c->bar, c->err, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   void* args[] = {(void*)&I, (void*)&c->bar, (void*)&c->err};
-  e = cudaLaunchCooperativeKernel((const void*)lhdm_solve_grid_kernel, dim3(c->nsm), dim3(NT), args, DYN_SMEM, st);
+  e = cudaLaunchCooperativeKernel((const void*)lhdm_solve_grid_kernel, dim3(c->ctas), dim3(NT), args, DYN_SMEM, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   c->have_state = p.mode == LHDM_MODE_NNLS;  // the adjoint covers problem (1) only
   c->last_m = m;
@@ -523,6 +525,14 @@ int lhdm_debug_commit_guard(lhdm_ctx* c, int32_t mode) {
 int lhdm_debug_inject(lhdm_ctx* c, int32_t what) {
   if (!c || (what & ~LHDM_INJECT_ALL)) return LHDM_ERR_INVALID_ARG;
   c->inject = what;
+  return LHDM_OK;
+}
+
+int lhdm_debug_set_ctas(lhdm_ctx* c, int32_t ctas) {
+  if (!c || ctas < 0 || ctas == 1 || ctas > c->nsm) return LHDM_ERR_INVALID_ARG;
+  const int t = ctas ? ctas : c->nsm;
+  if ((c->max_n + t - 1) / t > CAND_LOCAL_MAX) return LHDM_ERR_INVALID_ARG;
+  c->ctas = t;
   return LHDM_OK;
 }
 

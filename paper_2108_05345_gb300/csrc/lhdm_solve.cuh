@@ -2106,28 +2106,33 @@ struct Engine {
     for (int j = tid; j <= nrot; j += NT) sv[j] = ldcg(v + j);
     __syncthreads();
     int lo, hi;
-    split(nrot, tm.size, tm.rank, lo, hi);  // nrot <= INV_ROWS: at most 32 each
+    split(nrot, tm.size, tm.rank, lo, hi);
     if (lo < hi) {
       double b = 0.0;
       for (int j = tid; j <= lo; j += NT) b = fma(sv[j], sv[j], b);
       b = block_sum(b, sh);  // h_lo^2
       if (warp == 0) {
-        const int i = lo + lane;
-        const double vn = (i < hi) ? sv[i + 1] : 0.0;
-        double inc = vn * vn;
+        // one strip of 32 on a whole GPU (nrot <= INV_ROWS over 152 CTAs),
+        // several on a team of fewer CTAs
+        for (int i0 = lo; i0 < hi; i0 += 32) {
+          const int i = i0 + lane;
+          const double vn = (i < hi) ? sv[i + 1] : 0.0;
+          double inc = vn * vn;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += t;
-        }
-        const double h2 = b + inc;
-        double hp = __shfl_up_sync(0xffffffffu, h2, 1);
-        if (lane == 0) hp = b;
-        if (i < hi) {
-          const double ih = rsqrt(h2);
-          I.rotc[i] = vn * ih;
-          I.rots[i] = -(i == 0 ? sv[0] : sqrt_gm(hp)) * ih;
-          if (!(h2 < 0x1p+1000) || !(b > 0x1p-900)) I.ctl[C_DEL] = ep;
+          for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+          }
+          const double h2 = b + inc;
+          double hp = __shfl_up_sync(0xffffffffu, h2, 1);
+          if (lane == 0) hp = b;
+          if (i < hi) {
+            const double ih = rsqrt(h2);
+            I.rotc[i] = vn * ih;
+            I.rots[i] = -(i == 0 ? sv[0] : sqrt_gm(hp)) * ih;
+            if (!(h2 < 0x1p+1000) || !(b > 0x1p-900)) I.ctl[C_DEL] = ep;
+          }
+          b = __shfl_sync(0xffffffffu, h2, 31);
         }
       }
     }

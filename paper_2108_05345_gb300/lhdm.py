@@ -79,6 +79,7 @@ def lib():
         L.lhdm_debug_stall_next_solve.argtypes = [V]
         L.lhdm_debug_commit_guard.argtypes = [V, i32]
         L.lhdm_debug_inject.argtypes = [V, i32]
+        L.lhdm_debug_set_ctas.argtypes = [V, i32]
         L.lhdm_debug_fast_math.argtypes = [V, V, i32, V]
         L.lhdm_phase_times.argtypes = [V, C.POINTER(C.c_double), i32, V]
         L.lhdm_trace.argtypes = [V, C.POINTER(C.c_int32), i32, V]
@@ -354,6 +355,10 @@ class Context:
     def inject(self, what):
         """Failure-detection test aid (lhdm_debug_inject)."""
         _check(lib().lhdm_debug_inject(self.h, int(what)), "lhdm_debug_inject")
+
+    def set_ctas(self, ctas):
+        """Test aid: later solves run on that many CTAs (0: one per SM)."""
+        _check(lib().lhdm_debug_set_ctas(self.h, int(ctas)), "lhdm_debug_set_ctas")
 
     def stall_next_solve(self):
         _check(lib().lhdm_debug_stall_next_solve(self.h), "lhdm_debug_stall_next_solve")
