@@ -321,10 +321,14 @@ int lhdm_debug_commit_guard(lhdm_ctx* ctx, int32_t mode);
  * LHDM_INJECT_COMMIT_STALL: the tensor-core commit leaves out the last
  * arrivals its matrix products wait for; every wait of the commit runs out
  * (4 s), what was in flight is waited for, and the solve returns
- * LHDM_ERR_TIMEOUT; the context stays usable.  Errors: INVALID_ARG.
+ * LHDM_ERR_TIMEOUT; the context stays usable.  LHDM_INJECT_SOLVE_TEST: the
+ * solves of inner steps with the kept inverse of R fail their residual test,
+ * so the first one gives the inverse up (the deletions' own test stays as it
+ * is).  Errors: INVALID_ARG.
  */
 #define LHDM_INJECT_COMMIT_STALL 1
-#define LHDM_INJECT_ALL 1
+#define LHDM_INJECT_SOLVE_TEST 2
+#define LHDM_INJECT_ALL 3
 int lhdm_debug_inject(lhdm_ctx* ctx, int32_t what);
 
 /*
@@ -374,7 +378,7 @@ int lhdm_trace(lhdm_ctx* ctx, int32_t* out, int32_t max_rows, void* stream);
  * min(max_m, max_n) rounded up to even), "ctl" (16 int32 control words;
  * [10] = commit batches that the accuracy guard of the tensor-core commit
  * sent to FP64, [11] and [12] nonzero after a failed test of the kept
- * inverse).  FP64 except the int32 arrays.  Errors: INVALID_ARG for an unknown name or count too large. */
+ * inverse, [13] = deletions that took their rotations from it).  FP64 except the int32 arrays.  Errors: INVALID_ARG for an unknown name or count too large. */
 int lhdm_debug_state(lhdm_ctx* ctx, const char* name, void* host, int64_t count, void* stream);
 
 /* Profile of the last solve on ctx.  ms[0..12) = device time in ms of each

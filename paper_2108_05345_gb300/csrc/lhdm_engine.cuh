@@ -145,7 +145,8 @@ struct Inst {
 enum { C_KP = 0, C_DROPS, C_CAND, C_NROT, C_NRUN, C_READY, C_STATUS, C_ERR, C_KK, C_NFLIP,
        C_GUARD1,  // commit batches the accuracy guard handed to the FP64 path
        C_INV,     // last corrected solve whose residual test failed
-       C_DEL };   // last deletion whose rotations from the inverse failed their test
+       C_DEL,     // last deletion whose rotations from the inverse failed their test
+       C_NDEL };  // deletions that took their rotations from the inverse
 
 // ---------------------------------------------------------------- helpers
 __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }

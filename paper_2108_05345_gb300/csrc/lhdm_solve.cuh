@@ -2067,7 +2067,8 @@ struct Engine {
           I.rres[p0 + lane] = d;
           // |d| <= 2^-INV_BITS times the largest term (at least 2^(g - 2)); a
           // term that is not finite fails
-          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || (I.guard_force == 1 && inner_step > 0)) I.ctl[C_INV] = ep;
+          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || ((I.guard_force == 1 || (I.inject & LHDM_INJECT_SOLVE_TEST)) && inner_step > 0))
+            I.ctl[C_INV] = ep;
         }
       }
       __syncthreads();
@@ -2080,8 +2081,9 @@ struct Engine {
     const int ep = ++iepoch;
     inv_residual(np, ep);
     if (!sync()) return false;
-    if (ldcg(I.ctl + C_INV) == ep) {
+    if (ldcg(I.ctl + C_INV) == ep) {  // given up: for solves and for deletions
       inv_on = false;
+      inv_n = 0;
       return trsv(np);
     }
     inv_product(np, I.rres, true);
@@ -3574,12 +3576,13 @@ struct Engine {
     }
     if (!sync()) return false;
     phase(PH_CHAIN);
-    if (inv_n == np && nrot > 0) {
+    if (inv_on && inv_n == np && nrot > 0) {
       const int ep = ++iepoch;
       inv_rotations(q, np, nrot, ep);
       if (!sync()) return false;
       if (ldcg(I.ctl + C_DEL) != ep) {
         phase(PH_ZROT);
+        if (tm.rank == 0 && tid == 0) ++I.ctl[C_NDEL];
         nP = np - 1;
         rotate_columns(q, np, nrot, 0, false);
         inv_n = np - 1;
