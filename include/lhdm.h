@@ -324,11 +324,15 @@ int lhdm_debug_commit_guard(lhdm_ctx* ctx, int32_t mode);
  * LHDM_ERR_TIMEOUT; the context stays usable.  LHDM_INJECT_SOLVE_TEST: the
  * solves of inner steps with the kept inverse of R fail their residual test,
  * so the first one gives the inverse up (the deletions' own test stays as it
- * is).  Errors: INVALID_ARG.
+ * is).  LHDM_INJECT_CHECK_APPEND, LHDM_INJECT_CHECK_INNER: the same for the
+ * test of what such a solve returns, in appends and in inner steps.  Errors:
+ * INVALID_ARG.
  */
 #define LHDM_INJECT_COMMIT_STALL 1
 #define LHDM_INJECT_SOLVE_TEST 2
-#define LHDM_INJECT_ALL 3
+#define LHDM_INJECT_CHECK_APPEND 4
+#define LHDM_INJECT_CHECK_INNER 8
+#define LHDM_INJECT_ALL 15
 int lhdm_debug_inject(lhdm_ctx* ctx, int32_t what);
 
 /*
@@ -372,8 +376,8 @@ int lhdm_trace(lhdm_ctx* ctx, int32_t* out, int32_t max_rows, void* stream);
 
 /* Verification aid: copies `count` elements of a named piece of the
  * context's device state after the last solve to host memory `host`
- * (synchronises).  Names: "w", "u", "anorm" (length n), "bt", "r"
- * (length m), "yP", "xP", "order", "rslot" (positions), "pos" (columns),
+ * (synchronises).  Names: "w", "u", "anorm" (length n), "bt", "r",
+ * "rhs" (length m), "yP", "xP", "order", "rslot" (positions), "pos" (columns),
  * "W" (ld = max_m rounded up to even), "R" (slot-major, ld = the context's
  * min(max_m, max_n) rounded up to even), "ctl" (16 int32 control words;
  * [10] = commit batches that the accuracy guard of the tensor-core commit

@@ -401,6 +401,7 @@ int lhdm_debug_state(lhdm_ctx* c, const char* name, void* host, int64_t count, v
   const Entry table[] = {
       {"w", c->dscr + c->L.w, 8, n},          {"u", c->dscr + c->L.u, 8, n},
       {"anorm", c->dscr + c->L.anorm, 8, n},  {"bt", c->dscr + c->L.bt, 8, m},
+      {"rhs", c->dscr + c->L.rhs, 8, std::max(m, cp)},
       {"yP", c->dscr + c->L.yP, 8, cp},       {"xP", c->xP, 8, cp},
       {"r", c->r, 8, m},                      {"W", c->dscr + c->L.W, 8, (size_t)c->L.ldw * n},
       {"R", c->R, 8, (size_t)c->ldr * cp},    {"order", c->order, 4, cp},

@@ -1836,14 +1836,24 @@ struct Engine {
   // An append costs nP^2 k / 2 FMAs over the GPU, so the inverse is made when
   // an inner step first solves with more than INV_MIN positions (below, the
   // substitution is one or two blocks) or when k <= 3, and follows from there.
-  // Accuracy: the correction's residual is tested row by row against the
-  // row's largest |R| |y|: one product with the inverse leaves about
-  // |I - R R^{-1}| of it, the second the square of that, so 2^-26 guarantees
-  // rounding level.  Where a row misses it (R too ill-conditioned for an
-  // explicit inverse) the solve is done by substitution and the inverse is
-  // given up for the rest.
+  // Accuracy: what is accepted is tested.  The residual rhs - R y of the
+  // corrected y must be rounding, row by row: at most (16 + 8 min(k, 32)) 2^-53
+  // of the row's largest |R| |y| or of the row's sum |R y|, whichever is more,
+  // k the row's length (a substitution's own bound is k 2^-53 sum |R| |y|).
+  // Measured over uniform, conditioned (kappa 1e4 .. 1e13), nearly dependent
+  // and column-scaled instances with up to 1760 removals: at most 8 at k = 2,
+  // 27 at 8, 64 at 64 and 108 beyond.  The residual before the correction is
+  // only a rule for when to try: it says how far one product is off for this
+  // right-hand side, not what a second product does to it.  Where a row misses
+  // either (R too ill-conditioned for an explicit inverse) the solve is done
+  // by substitution and the inverse is given up for the rest.  The second test
+  // runs beside the commit (an append), beside rank 0's x update (an inner
+  // step) or, with a barrier of its own, at the end of the inner loop; it
+  // costs 2.4 % of a one-column solve at 2048 x 1024 (57.7 -> 59.2 ms) and of
+  // a conditioned one (52.9 -> 54.2 ms), 0.9 % at 4096 x 2048.
   static constexpr int INV_MIN = 2 * TB, INV_ROWS = 3072;
   static constexpr int INV_BITS = 26;
+  int chk_ep = 0;  // the corrected solve whose test is still to be read (0: none)
   __device__ __forceinline__ double* Irow(int p) const { return I.Rinv + (size_t)ldcg(I.rslot + p) * I.ldr; }
 
   // yP (+)= R^{-1} v on positions [0, np), a warp per row.
@@ -2007,23 +2017,26 @@ struct Engine {
     __syncthreads();  // the first append goes on to the commit, which overwrites dyn, without a team barrier
   }
 
-  // Residual rhs - R yP on rows [0, np) into rres, eight rows per CTA and
-  // pass (lanes: 8 rows x 4 columns), with the accuracy test.
-  __device__ void inv_residual(int np, int ep) {
+  // Residual rhs - R yP on rows [0, np), eight rows per CTA and pass (lanes:
+  // 8 rows x 4 columns), on ranks r0 up.  fin: the test of a corrected yP;
+  // else the residual goes into rres, with the test whether to correct.  A
+  // failed test (force: every test) leaves ep in the control word (a barrier
+  // must follow).
+  __device__ void inv_residual(int np, int ep, bool fin, int r0, bool force) {
     double* sy = dyn;                                    // np
     int* ss = reinterpret_cast<int*>(dyn + np);          // np
     double* sa = dyn + np + (np + 1) / 2;                // NW x 8
     int* sf = reinterpret_cast<int*>(sa + NW * 8);       // NW x 8
-    if (tm.rank * 8 >= np) return;
+    const int first = (tm.rank - r0) * 8, step = (tm.size - r0) * 8;
+    if (first < 0 || first >= np) return;
     __syncthreads();
-    const int first = tm.rank * 8;
     for (int c = first + tid; c < np; c += NT) {
       sy[c] = ldcg(I.yP + c);
       ss[c] = ldcg(I.rslot + c);
     }
     __syncthreads();
     const int row = lane & 7, cg = lane >> 3;
-    for (int p0 = first; p0 < np; p0 += tm.size * 8) {
+    for (int p0 = first; p0 < np; p0 += step) {
       double a = 0.0;
       int f = -8000;  // largest exponent of |R| |y| (a conversion to float is an FP64 instruction)
       const int r = min(p0 + row, np - 1);
@@ -2064,11 +2077,17 @@ struct Engine {
         g = max(g, __shfl_xor_sync(0xffffffffu, g, 16));
         if (lane < 8 && p0 + lane < np) {
           const double d = ldcg(I.rhs + p0 + lane) - t;
-          I.rres[p0 + lane] = d;
-          // |d| <= 2^-INV_BITS times the largest term (at least 2^(g - 2)); a
-          // term that is not finite fails
-          if (!isfinite(d) || ebound(d) > g - 2 - INV_BITS || ((I.guard_force == 1 || (I.inject & LHDM_INJECT_SOLVE_TEST)) && inner_step > 0))
-            I.ctl[C_INV] = ep;
+          // the largest term is at least 2^(g - 2); a row without one
+          // (all of yP zero there) needs a residual of zero
+          bool bad = d != 0.0;
+          if (fin) {
+            const double scale = fmax(fabs(t), pow2n(max(-1000, min(g - 2, 1023))));
+            if (g > -900) bad = !(fabs(d) <= (double)(16 + 8 * min(np - p0 - lane, 32)) * 0x1p-53 * scale);
+          } else {
+            I.rres[p0 + lane] = d;
+            if (g > -900) bad = !isfinite(d) || ebound(d) > g - 2 - INV_BITS;
+          }
+          if (bad || force) I.ctl[C_INV] = ep;
         }
       }
       __syncthreads();
@@ -2077,17 +2096,33 @@ struct Engine {
 
   // R y = rhs on [0, np) with yP already R^{-1} rhs (a barrier must have
   // followed): the correction, or the substitution where the test fails.
+  // After a correction the caller runs inv_check and, a barrier later,
+  // inv_settle.
   __device__ bool inv_correct(int np) {
     const int ep = ++iepoch;
-    inv_residual(np, ep);
+    inv_residual(np, ep, false, 0, (I.guard_force == 1 || (I.inject & LHDM_INJECT_SOLVE_TEST)) && inner_step > 0);
     if (!sync()) return false;
-    if (ldcg(I.ctl + C_INV) == ep) {  // given up: for solves and for deletions
-      inv_on = false;
-      inv_n = 0;
-      return trsv(np);
-    }
+    if (ldcg(I.ctl + C_INV) == ep) return inv_give_up(np);
     inv_product(np, I.rres, true);
+    chk_ep = ++iepoch;
     return sync();
+  }
+  // for solves and for deletions
+  __device__ bool inv_give_up(int np) {
+    inv_on = false;
+    inv_n = 0;
+    return trsv(np);
+  }
+  // The test of the corrected yP, on ranks r0 up (inject: the bit that fails it).
+  __device__ void inv_check(int np, int r0, int inject) {
+    if (chk_ep) inv_residual(np, chk_ep, true, r0, (I.inject & inject) != 0);
+  }
+  // Whether that test passed (every thread, after the barrier that follows
+  // inv_check); the substitution is the caller's where it failed.
+  __device__ bool inv_settle() {
+    const bool good = !chk_ep || ldcg(I.ctl + C_INV) != chk_ep;
+    chk_ep = 0;
+    return good;
   }
   // Rotations of the downdate that deletes position q, from row q of the kept
   // inverse (v, in the slot of the removed column).  v^T R~ = 0 for R without
@@ -3446,9 +3481,17 @@ struct Engine {
       // any y_P <= 0 ?  (with the positivity trick: y of the signed column)
       int neg = 0;
       for (int p = tid; p < nP; p += NT) neg |= (pos_sign(p) * ldcg(I.yP + p) <= 0.0);
-      if (!__syncthreads_or(neg)) return true;
-      if (steps > nP + 1) {
-        status = LHDM_ERR_MAX_ITER;
+      neg = __syncthreads_or(neg);
+      if (!neg || steps > nP + 1) {
+        if (chk_ep) {  // the test of the last solve
+          inv_check(nP, 0, LHDM_INJECT_CHECK_INNER);
+          if (!sync()) return false;
+          if (!inv_settle()) {
+            if (!inv_give_up(nP)) return false;
+            continue;
+          }
+        }
+        if (neg) status = LHDM_ERR_MAX_ITER;
         return true;
       }
       ++steps;
@@ -3486,7 +3529,7 @@ struct Engine {
             const int k = atomicAdd(&s_nq, 1);
             qlist[k] = p;
           }
-          I.xP[p] = xn;
+          (chk_ep ? I.rres : I.xP)[p] = xn;
         }
         __syncthreads();
         if (tid == 0) {
@@ -3501,7 +3544,21 @@ struct Engine {
           I.ctl[C_NRUN] = nq;
         }
       }
+      // the other ranks test the last solve meanwhile; x is kept aside until
+      // the test is read
+      const bool pending = chk_ep != 0;
+      if (pending) inv_check(nP, 1, LHDM_INJECT_CHECK_INNER);
       if (!sync()) return false;
+      if (!inv_settle()) {
+        --steps;
+        --n_inner;
+        if (!inv_give_up(nP)) return false;
+        continue;
+      }
+      if (pending && tm.rank == 0) {
+        for (int p = tid; p < nP; p += NT) I.xP[p] = ldcg(I.rres + p);
+        __syncthreads();
+      }
       const int nq = ldcg(I.ctl + C_NRUN);
       removed += nq;
       ++inner_step;
@@ -4655,7 +4712,10 @@ struct Engine {
         if (!trsv(nP)) return fail_out();
       }
       phase(PH_COMMIT);
+      const int np0 = nP;
+      inv_check(np0, 0, LHDM_INJECT_CHECK_APPEND);
       if (!commit(s_J)) return fail_out();
+      if (!inv_settle() && !inv_give_up(np0)) return fail_out();
       phase(PH_INNER);
       removed = 0;
       inner_step = 0;

@@ -26,6 +26,8 @@ LHDM_ERR_NO_STATE = 8
 LHDM_ERR_TOO_LARGE = 9
 LHDM_INJECT_COMMIT_STALL = 1
 LHDM_INJECT_SOLVE_TEST = 2
+LHDM_INJECT_CHECK_APPEND = 4
+LHDM_INJECT_CHECK_INNER = 8
 KMAX_LIMIT = 64
 MODE_NNLS, MODE_SIGNED, MODE_SIGNED_FLIP = 0, 1, 2
 PHASES = ("setup", "dm", "panel", "solve", "commit", "inner", "residual", "dual",
