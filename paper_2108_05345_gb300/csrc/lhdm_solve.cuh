@@ -2133,8 +2133,12 @@ struct Engine {
   // below the diagonal of column t is e_t = v(q .. t+1)^T R~_t / h_{t+1}, about
   // eps |R~_t| as the inverse is kept by row operations (a small residual
   // X R - I row by row); it is formed for every column, and where one is above
-  // 2^-47 |a_t| the chain takes the deletion and the inverse is given up.
-  static constexpr double DEL_TOL2 = 0x1p-94;
+  // 2^-49 |a_t| the chain takes the deletion and the inverse is given up.
+  // 2^-49 is 16 2^-53: a rotation's own rounding may be 6 2^-53 of a column,
+  // and a column takes one per position.  Measured in units of 2^-53: up to 1
+  // for uniform instances, 7, 8, 11, 14 and 27 for kappa = 1e4, 1e6, 1e8, 1e10
+  // and 1e13 (2048 x 1024, 421 to 1656 deletions a solve).
+  static constexpr double DEL_TOL2 = 0x1p-98;
   __device__ void inv_rotations(int q, int np, int nrot, int ep) {
     double* sv = dyn;  // v(q .. np - 1)
     __shared__ double sh[32];
