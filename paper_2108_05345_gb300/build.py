@@ -1,6 +1,6 @@
 """Builds the CUDA library liblhdm.so in-tree for sm_103a (GB300) with nvcc.
 
-Four translation units (the host side of the C ABI and one per kernel
+Six translation units (the host side of the C ABI and one per kernel
 family) compile in parallel and link into one shared library, which sits
 next to this file and is what paper_2108_05345_gb300.lhdm loads.
 """
@@ -13,7 +13,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "liblhdm.so")
-SOURCES = ["lhdm_api.cu", "lhdm_grid_solve.cu", "lhdm_batch_solve.cu", "lhdm_backward.cu"]
+SOURCES = ["lhdm_api.cu", "lhdm_grid_solve.cu", "lhdm_grid_solve_tall.cu", "lhdm_batch_solve.cu",
+           "lhdm_batch_solve_tall.cu", "lhdm_backward.cu"]
 HEADERS = ["lhdm_engine.cuh", "lhdm_solve.cuh", "lhdm_adjoint.cuh", "lhdm_kernels.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]

@@ -72,6 +72,7 @@ struct lhdm_batch {
   int device = 0;
   int batch = 0;
   int nblocks = 0;
+  bool tall = false;  // an instance has more than TALL_ROWS rows
   ScratchLayout L{};
   double* dscr = nullptr;
   int* iscr = nullptr;
@@ -111,7 +112,11 @@ static int set_attrs() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lhdm_backward_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN_SMEM);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(lhdm_solve_grid_tall_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN_SMEM);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lhdm_solve_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(lhdm_solve_batch_tall_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lhdm_backward_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN_SMEM);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
@@ -313,7 +318,8 @@ int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, 
   cudaError_t e = clear_words(c->bar, c->err, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   void* args[] = {(void*)&I, (void*)&c->bar, (void*)&c->err};
-  e = cudaLaunchCooperativeKernel((const void*)lhdm_solve_grid_kernel, dim3(c->ctas), dim3(NT), args, DYN_SMEM, st);
+  const void* kernel = m > TALL_ROWS ? (const void*)lhdm_solve_grid_tall_kernel : (const void*)lhdm_solve_grid_kernel;
+  e = cudaLaunchCooperativeKernel(kernel, dim3(c->ctas), dim3(NT), args, DYN_SMEM, st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   c->have_state = p.mode == LHDM_MODE_NNLS;  // the adjoint covers problem (1) only
   c->last_m = m;
@@ -735,6 +741,7 @@ int lhdm_batch_create(lhdm_batch** out, int32_t batch, const int32_t* m, const i
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, B->device);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lhdm_solve_batch_kernel, NT, DYN_SMEM);
   B->batch = batch;
+  B->tall = max_m > TALL_ROWS;
   B->nblocks = std::max(1, std::min(batch, nsm * std::max(occ, 1)));
   B->L = make_layout(max_m, max_n, 1);
   B->prm = to_dev(p);
@@ -815,8 +822,8 @@ int lhdm_batch_run(lhdm_batch* B, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemsetAsync(B->d_queue, 0, sizeof(int), st);
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
-  lhdm_solve_batch_kernel<<<B->nblocks, NT, DYN_SMEM, st>>>(B->d_items, B->d_perm, B->batch, B->d_queue, B->L,
-                                                             B->dscr, B->iscr, B->prm);
+  const auto kernel = B->tall ? lhdm_solve_batch_tall_kernel : lhdm_solve_batch_kernel;
+  kernel<<<B->nblocks, NT, DYN_SMEM, st>>>(B->d_items, B->d_perm, B->batch, B->d_queue, B->L, B->dscr, B->iscr, B->prm);
   e = cudaGetLastError();
   if (e != cudaSuccess) return LHDM_ERR_CUDA;
   B->ran = true;

@@ -1,0 +1,12 @@
+// lhdm_batch_solve_tall.cu -- the persistent solve kernel of a batch of instances with
+// tall ones among them.
+#include "lhdm_kernels.cuh"
+
+using namespace lhdm;
+
+__global__ void __launch_bounds__(NT, 1) lhdm_solve_batch_tall_kernel(const BatchItem* items, const int* perm,
+                                                                      int batch, int* queue, ScratchLayout L,
+                                                                      double* dscr, int* iscr, DevParams prm) {
+  extern __shared__ double dyn[];
+  solve_queue<true>(items, perm, batch, queue, L, dscr, iscr, prm, dyn);
+}

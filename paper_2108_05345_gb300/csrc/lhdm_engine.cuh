@@ -633,7 +633,7 @@ __device__ __forceinline__ bool wait_ge(const int* flag, int target, int* err, l
   return true;
 }
 
-template <class Team>
+template <class Team, bool TALL = false>
 struct Engine;
 
 }  // namespace lhdm

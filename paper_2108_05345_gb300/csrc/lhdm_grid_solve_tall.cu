@@ -1,0 +1,9 @@
+// lhdm_grid_solve_tall.cu -- the solve kernel of one tall instance on the whole GPU.
+#include "lhdm_kernels.cuh"
+
+using namespace lhdm;
+
+__global__ void __launch_bounds__(NT, 1) lhdm_solve_grid_tall_kernel(Inst I, unsigned int* bar, int* err) {
+  extern __shared__ double dyn[];
+  solve_on_grid<true>(I, bar, err, dyn);
+}

@@ -1,8 +1,8 @@
 // lhdm_kernels.cuh -- what the kernels and the host side of the C ABI
 // share: the batch descriptor, the scratch layout and the kernel
 // declarations.  Each kernel is compiled in a translation unit of its own
-// (lhdm_grid_solve.cu, lhdm_batch_solve.cu, lhdm_backward.cu) so the library
-// builds in parallel.
+// (lhdm_grid_solve.cu, lhdm_batch_solve.cu, their _tall forms,
+// lhdm_backward.cu) so the library builds in parallel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -205,19 +205,77 @@ inline __device__ void bind_item(Inst& I, const BatchItem& it) {
   I.prm.k_max = it.k_max;
 }
 
+// One solve on the whole GPU.
+template <bool TALL>
+__device__ __forceinline__ void solve_on_grid(const Inst& I, unsigned int* bar, int* err, double* dyn) {
+  GridTeam tm{(int)blockIdx.x, (int)gridDim.x, bar, err, I.wait_ns, I.bar_extra};
+  Engine<GridTeam, TALL> e(tm, I, dyn);
+  const TcState tc = tc_open();
+  e.mbs = tc.mbs;
+  e.tmem = tc.tmem;
+  e.run();
+  tc_close(tc);
+}
+
+// Many instances in one persistent launch: each CTA takes the next instance
+// (largest first) from a device queue and solves it alone.
+template <bool TALL>
+__device__ __forceinline__ void solve_queue(const BatchItem* items, const int* perm, int batch, int* queue,
+                                            const ScratchLayout& L, double* dscr, int* iscr, const DevParams& prm,
+                                            double* dyn) {
+  __shared__ int s_k;
+  Inst I;
+  bind_scratch(I, L, dscr + (size_t)blockIdx.x * L.dtotal, iscr + (size_t)blockIdx.x * L.itotal);
+  I.phase_ns = nullptr;
+  I.trace = nullptr;
+  I.trace_cap = 0;
+  const TcState tc = tc_open();
+  unsigned mpar = 0u;  // parities of tc's barriers, from instance to instance
+  for (;;) {
+    if (threadIdx.x == 0) s_k = atomicAdd(queue, 1);
+    __syncthreads();
+    const int k = s_k;
+    __syncthreads();
+    if (k >= batch) break;
+    const BatchItem it = items[perm[k]];
+    I.prm = prm;
+    bind_item(I, it);
+    CtaTeam tm{0, 1};
+    Engine<CtaTeam, TALL> e(tm, I, dyn);
+    e.mbs = tc.mbs;
+    e.tmem = tc.tmem;
+    e.mpar = mpar;
+    e.run();
+    mpar = e.mpar;
+    if (e.tc_failed) {
+      tc_reset(tc);
+      mpar = 0u;
+    }
+    __syncthreads();
+  }
+  tc_close(tc);
+}
+
 }  // namespace lhdm
 
-// One solve on the whole GPU: one CTA per SM, cooperative launch.
+// One solve on the whole GPU: one CTA per SM, cooperative launch; the second
+// for more than TALL_ROWS rows.
 __global__ void __launch_bounds__(lhdm::NT, 1) lhdm_solve_grid_kernel(lhdm::Inst I, unsigned int* bar, int* err);
+__global__ void __launch_bounds__(lhdm::NT, 1) lhdm_solve_grid_tall_kernel(lhdm::Inst I, unsigned int* bar, int* err);
 // Adjoint of a solve on the whole GPU (cooperative launch).
 __global__ void __launch_bounds__(lhdm::NT, 1) lhdm_backward_grid_kernel(lhdm::Inst I, unsigned int* bar, int* err,
                                                                          const double* g, double* dLdb,
                                                                          double* dLdA, int ld_dA, double* apu);
-// Many instances in one persistent launch, one instance per CTA at a time.
+// Many instances in one persistent launch, one instance per CTA at a time; the
+// second when any has more than TALL_ROWS rows.
 __global__ void __launch_bounds__(lhdm::NT, 1) lhdm_solve_batch_kernel(const lhdm::BatchItem* items,
                                                                        const int* perm, int batch, int* queue,
                                                                        lhdm::ScratchLayout L, double* dscr,
                                                                        int* iscr, lhdm::DevParams prm);
+__global__ void __launch_bounds__(lhdm::NT, 1) lhdm_solve_batch_tall_kernel(const lhdm::BatchItem* items,
+                                                                            const int* perm, int batch, int* queue,
+                                                                            lhdm::ScratchLayout L, double* dscr,
+                                                                            int* iscr, lhdm::DevParams prm);
 __global__ void __launch_bounds__(lhdm::NT, 1) lhdm_backward_batch_kernel(const lhdm::BatchItem* items,
                                                                           const int* perm, int batch, int* queue,
                                                                           lhdm::ScratchLayout L, double* dscr,

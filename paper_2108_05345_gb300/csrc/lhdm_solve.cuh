@@ -11,6 +11,9 @@ constexpr int DYN_SMEM = 164 * 1024;
 constexpr int CAND_LOCAL_MAX = 2048;     // local DM candidates per CTA
 constexpr int CAND_STAGE = 4096;         // merged candidates staged per pass
 constexpr int ROT_STAGE = 2048;          // rotations staged per pass
+// Beyond, the rows of four reflectors do not fit a commit's work area (five and
+// more reflectors take the tensor cores up to 16384 rows).
+constexpr int TALL_ROWS = (DYN_SMEM / 8 - 2 * KM * 16) / 4;
 
 // Orderable key of a positive double (dual values of DM candidates are > 0).
 __device__ __forceinline__ unsigned long long wkey(double v) {
@@ -21,7 +24,10 @@ __device__ __forceinline__ bool better(unsigned long long ka, int ia, unsigned l
   return ka > kb || (ka == kb && ia < ib);
 }
 
-template <class Team>
+// TALL: with the commit's form for instances of more than TALL_ROWS rows (an
+// engine of its own, as that form's registers cost every phase of the others
+// 1 to 3 %).
+template <class Team, bool TALL>
 struct Engine {
   Team& tm;
   const Inst& I;
@@ -2294,6 +2300,7 @@ struct Engine {
     const int* s_cid;  // batch columns (-1: b)
   };
   static constexpr int CB = 16;  // Z columns per commit batch
+  static constexpr int WKD = DYN_SMEM / 8 - 2 * KM * CB;  // a commit's work area, in doubles
 
   __device__ __forceinline__ double* commit_col(const int* s_cid, int k) const {
     const int id = s_cid[k];
@@ -2322,15 +2329,16 @@ struct Engine {
   // broadcast or 32 consecutive doubles, so it runs at the FP64 pipe's rate:
   // about kp L 32 cycles per 32 columns (two lane FMAs a cycle) and 4000
   // beside them.  Every sum runs in an order fixed by kp and L.
+  static constexpr int XS = 33;
+  __device__ __forceinline__ int cols_rows() const { return (DYN_SMEM / 8 - (2 * kp + NW) * XS) / ((kp | 1) + XS); }
   __device__ void commit_cols(const double* s_T, const double* s_vt, const int* list, int n, int L) {
-    constexpr int XS = 33;
     const int VS = kp | 1;
     double* sD = dyn;                    // kp x XS, then D'
     double* sE = sD + kp * XS;
     double* sN = sE + kp * XS;           // NW x XS
     double* wk = sN + NW * XS;
     const int room = DYN_SMEM / 8 - (2 * kp + NW) * XS;
-    const bool whole = L <= room / (VS + XS);
+    const bool whole = L <= cols_rows();
     const int RC = whole ? L : (room / (VS + XS)) & ~31;
     const bool two = whole && L * (VS + 2 * XS) <= room;
     double* sV = wk;
@@ -2516,6 +2524,170 @@ struct Engine {
       if (list[tid] >= 0) I.u[list[tid]] = sqrt(v);
     }
     __syncthreads();
+  }
+
+  // Rows [rb, rb+nr) of V (kp columns) into the work area with row stride VS.
+  __device__ __forceinline__ void stage_vchunk(double* wk, int VS, const double* s_vt, int rb, int nr) {
+    const int tot = nr * kp;
+    for (int e0 = tid; e0 < tot; e0 += 4 * NT) {
+      double v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int e = e0 + k * NT, rr = e / kp, t = e - rr * kp, rg = rb + rr;
+        v[k] = (e < tot && rg > t) ? ldcg(I.V + (size_t)rg * KM + t) : ((e < tot && rg == t) ? s_vt[t] : 0.0);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int e = e0 + k * NT, rr = e / kp, t = e - rr * kp;
+        if (e < tot) wk[rr * VS + t] = v[k];
+      }
+    }
+  }
+
+  // One batch of NB columns in FP64: D = V^T C (pass 1: thread (t1, g1) sums rows
+  // g1, g1+G, ... of every chunk, then a fixed pairwise tree over g1),
+  // D' = T^T D, C -= V D' and the trailing norms (pass 2: thread (r2, grp)
+  // updates row r2 of every chunk in columns grp, grp+NG, ...).  It takes the
+  // columns of tall instances: a value of V is loaded once for NB FMAs and no
+  // lane is left without a column, where commit_cols works on 32 columns
+  // whatever a CTA has.  Commit phase against commit_cols over chunks of
+  // rows: 20000 x 300, k_max 8 9.4 ms (111); 20000 x 1000, k_max 32 46 (276);
+  // 24000 x 4096, k_max 32 706 (1214); 8000 x 1000, k_max 4 23.5 (143).
+  template <int NB>
+  __device__ __forceinline__ void commit_batch(const CommitShape& cs) {
+    const int L = cs.L, VS = kp | 1;
+    const int RC1 = min(1024, (WKD / (VS + CB)) & ~31);  // pass-1 rows per chunk
+    const int RC2 = WKD / VS >= 512 ? 512 : 256;         // VS <= 65
+    double* wk = dyn + 2 * KM * CB;
+    double* s_nrm = cs.s_D;  // NW x CB, once D is read
+    const int G = NT / kp, t1 = tid % kp, g1 = tid / kp;
+    const bool act1 = g1 < G;
+    double acc[NB];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) acc[c] = 0.0;
+    double* sX = wk + RC1 * VS;  // NB x RC1
+    for (int rb = 0; rb < L; rb += RC1) {
+      const int nr = min(RC1, L - rb);
+      __syncthreads();
+      stage_vchunk(wk, VS, cs.s_vt, rb, nr);
+      const int totx = NB * nr;
+      for (int e0 = tid; e0 < totx; e0 += 4 * NT) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int e = e0 + k * NT, cc = e / nr, rr = e - cc * nr;
+          v[k] = (e < totx) ? ldcg(commit_col(cs.s_cid, cc) + rb + rr) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int e = e0 + k * NT, cc = e / nr, rr = e - cc * nr;
+          if (e < totx) sX[cc * RC1 + rr] = v[k];
+        }
+      }
+      __syncthreads();
+      if (act1) {
+        for (int rr = g1; rr < nr; rr += G) {
+          const double v = wk[rr * VS + t1];
+#pragma unroll
+          for (int c = 0; c < NB; ++c) acc[c] = fma(v, sX[c * RC1 + rr], acc[c]);
+        }
+      }
+    }
+    __syncthreads();
+    double* P = wk;  // G x kp x NB partials
+    if (act1) {
+#pragma unroll
+      for (int c = 0; c < NB; ++c) P[(g1 * kp + t1) * NB + c] = acc[c];
+    }
+    __syncthreads();
+    for (int st = 1; st < G; st <<= 1) {
+      if (act1 && (g1 & (2 * st - 1)) == 0 && g1 + st < G) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) P[(g1 * kp + t1) * NB + c] += P[((g1 + st) * kp + t1) * NB + c];
+      }
+      __syncthreads();
+    }
+    for (int o = tid; o < kp * NB; o += NT) {
+      const int t = o / NB, cc = o - t * NB;
+      cs.s_D[t * CB + cc] = P[t * NB + cc];
+    }
+    __syncthreads();
+    // D' = T^T D
+    for (int o = tid; o < kp * NB; o += NT) {
+      const int t = o % kp, cc = o / kp;
+      double e2 = 0.0;
+      for (int sidx = 0; sidx <= t; ++sidx) e2 = fma(cs.s_T[t * (t + 1) / 2 + sidx], cs.s_D[sidx * CB + cc], e2);
+      cs.s_E[t * CB + cc] = e2;
+    }
+    // pass 2 (NG = 1 or 2 groups of columns)
+    const int NG = NT / RC2, r2 = tid % RC2, grp = tid / RC2;
+    constexpr int NK2 = (NB + 1) / 2;
+    double nrm[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) nrm[k] = 0.0;
+    for (int rb = 0; rb < L; rb += RC2) {
+      const int nr = min(RC2, L - rb);
+      __syncthreads();
+      stage_vchunk(wk, VS, cs.s_vt, rb, nr);
+      __syncthreads();
+      if (r2 < nr) {
+        const bool below = rb + r2 >= kp;
+        if (NG == 1) {
+          double x[NB];
+#pragma unroll
+          for (int k = 0; k < NB; ++k) x[k] = ldcg(commit_col(cs.s_cid, k) + rb + r2);
+          for (int t = 0; t < kp; ++t) {
+            const double v = wk[r2 * VS + t];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) x[k] = fma(-v, cs.s_E[t * CB + k], x[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < NB; ++k) {
+            commit_col(cs.s_cid, k)[rb + r2] = x[k];
+            if (below) nrm[k] = fma(x[k], x[k], nrm[k]);
+          }
+        } else {
+          double x[NK2];
+#pragma unroll
+          for (int k = 0; k < NK2; ++k) {
+            const int c = grp + 2 * k;
+            x[k] = (c < NB) ? ldcg(commit_col(cs.s_cid, c) + rb + r2) : 0.0;
+          }
+          for (int t = 0; t < kp; ++t) {
+            const double v = wk[r2 * VS + t];
+#pragma unroll
+            for (int k = 0; k < NK2; ++k) {
+              const int c = grp + 2 * k;
+              if (c < NB) x[k] = fma(-v, cs.s_E[t * CB + c], x[k]);
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < NK2; ++k) {
+            const int c = grp + 2 * k;
+            if (c < NB) {
+              commit_col(cs.s_cid, c)[rb + r2] = x[k];
+              if (below) nrm[k] = fma(x[k], x[k], nrm[k]);
+            }
+          }
+        }
+      }
+    }
+    // norms: a group's threads are whole warps; column c = grp + NG k
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const int c = grp + NG * k;
+      if (c < NB) {
+        const double v = warp_sum(nrm[k]);
+        if (lane == 0) s_nrm[warp * CB + c] = v;
+      }
+    }
+    __syncthreads();
+    if (tid < NB) {
+      const int g = tid % NG, w0 = g * (RC2 / 32);
+      double v = 0.0;
+      for (int w2 = 0; w2 < RC2 / 32; ++w2) v += s_nrm[(w0 + w2) * CB + tid];
+      if (cs.s_cid[tid] >= 0) I.u[cs.s_cid[tid]] = sqrt(v);
+    }
   }
 
   // One batch of nb <= NB (8 or 16) columns through the tensor cores, for
@@ -3389,8 +3561,7 @@ struct Engine {
     }
     double* s_D = dyn;                              // KM x CB
     double* s_E = dyn + KM * CB;                    // KM x CB
-    double* wk = dyn + 2 * KM * CB;                 // work area
-    constexpr int WKD = DYN_SMEM / 8 - 2 * KM * CB; // its size in doubles
+    double* wk = dyn + 2 * KM * CB;                 // WKD doubles
     __shared__ double s_T[KM * KM / 2 + KM];
     __shared__ double s_vt[KM];
     __shared__ int s_cid[CB];
@@ -3422,12 +3593,13 @@ struct Engine {
     const bool fits = (size_t)L * ((kp | 1) + nl) + 2 * KM * 8 + 32 <= DYN_SMEM / 8;
     const int nb16 = (nl + CB - 1) / CB, nb32 = (nl + 31) / 32;
     const float tc_cost = nl <= 8 ? 30000.f + 30.f * L : nb16 * (30000.f + 60.f * L);
+    const bool tall = TALL && I.m > TALL_ROWS;
     const bool test = I.guard_force != 0;  // the guard's test: the tensor-core form wherever it can run
     const bool narrow = nl <= 8 && fits && (!can || (!test && (float)kp * L * nl + 8000.f < tc_cost));
     const bool tc = can && !narrow && (test || nl <= 8 || tc_cost < nb32 * ((float)kp * L * 32.f + 6000.f));
     if (narrow) {
       commit_narrow(s_T, s_vt, s_list, nl, L);
-    } else if (!tc) {
+    } else if (!tc && !(tall && L > cols_rows())) {
       commit_cols(s_T, s_vt, s_list, nl, L);
     } else {
       for (int base = 0; base < nl; base += CB) {
@@ -3435,12 +3607,38 @@ struct Engine {
         __syncthreads();
         if (tid < nb) s_cid[tid] = s_list[base + tid];
         __syncthreads();
-        const int r = (nb <= 8) ? commit_tc<8>(cs, nb) : commit_tc<16>(cs, nb);
+        int r = 2;
+        if (!TALL || tc) r = (nb <= 8) ? commit_tc<8>(cs, nb) : commit_tc<16>(cs, nb);
         if (r == 1) {
           tc_failed = true;
           return false;
         }
-        if (r == 2) commit_cols(s_T, s_vt, s_list + base, nb, L);  // handed over by the accuracy guard
+        if (r == 0) continue;
+        // handed over by the accuracy guard, or a tall instance
+        if constexpr (TALL) {
+          if (tall) {
+            switch (nb) {
+              case 1: commit_batch<1>(cs); break;
+              case 2: commit_batch<2>(cs); break;
+              case 3: commit_batch<3>(cs); break;
+              case 4: commit_batch<4>(cs); break;
+              case 5: commit_batch<5>(cs); break;
+              case 6: commit_batch<6>(cs); break;
+              case 7: commit_batch<7>(cs); break;
+              case 8: commit_batch<8>(cs); break;
+              case 9: commit_batch<9>(cs); break;
+              case 10: commit_batch<10>(cs); break;
+              case 11: commit_batch<11>(cs); break;
+              case 12: commit_batch<12>(cs); break;
+              case 13: commit_batch<13>(cs); break;
+              case 14: commit_batch<14>(cs); break;
+              case 15: commit_batch<15>(cs); break;
+              default: commit_batch<16>(cs); break;
+            }
+            continue;
+          }
+        }
+        commit_cols(s_T, s_vt, s_list + base, nb, L);
       }
     }
     nP += kp;
@@ -4367,7 +4565,10 @@ struct Engine {
     return true;
   }
 
-  __device__ int* tm_err();
+  __device__ __forceinline__ int* tm_err() {
+    if constexpr (std::is_same<Team, GridTeam>::value) return tm.err;
+    else return nullptr;
+  }
 
   // ------------------------------------------------------------ residual and dual
   // r = b - A_P x_P (row tiles of 32 rows, warps split the positions).
@@ -4769,10 +4970,5 @@ struct Engine {
     }
   }
 };
-
-template <>
-__device__ __forceinline__ int* Engine<GridTeam>::tm_err() { return tm.err; }
-template <>
-__device__ __forceinline__ int* Engine<CtaTeam>::tm_err() { return nullptr; }
 
 }  // namespace lhdm
