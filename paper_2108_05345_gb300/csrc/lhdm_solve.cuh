@@ -2321,17 +2321,18 @@ struct Engine {
     }
   }
 
-  // FP64 commit of n columns, 32 at a time with a lane per column: D = V^T C
-  // (a warp per reflector), D' = T^T D, C -= V D' and the trailing norms (a
-  // warp per row).  V and the columns' rows are staged in shared memory, all
-  // of them when they fit, else RC at a time; the next 32 columns are copied
+  // FP64 commit of n columns, CW = 2^lw at a time with a lane per column (and
+  // 32 / CW rows side by side): D = V^T C (a warp per reflector), D' = T^T D,
+  // C -= V D' and the trailing norms (a warp per row).  V and the columns' rows are staged in shared memory, all
+  // of them when they fit, else RC at a time; the next CW columns are copied
   // meanwhile when a second buffer fits.  Every operand of an FMA is a
-  // broadcast or 32 consecutive doubles, so it runs at the FP64 pipe's rate:
-  // about kp L 32 cycles per 32 columns (two lane FMAs a cycle) and 4000
-  // beside them.  Every sum runs in an order fixed by kp and L.
+  // broadcast or consecutive doubles, so it runs at the FP64 pipe's rate:
+  // about kp L CW cycles per CW columns (two lane FMAs a cycle) and 4000
+  // beside them.  Every sum runs in an order fixed by kp, L and CW.
   static constexpr int XS = 33;
   __device__ __forceinline__ int cols_rows() const { return (DYN_SMEM / 8 - (2 * kp + NW) * XS) / ((kp | 1) + XS); }
-  __device__ void commit_cols(const double* s_T, const double* s_vt, const int* list, int n, int L) {
+  __device__ void commit_cols(const double* s_T, const double* s_vt, const int* list, int n, int L, int lw) {
+    const int CW = 1 << lw, G = 32 >> lw, cl = lane & (CW - 1), g = lane >> lw;
     const int VS = kp | 1;
     double* sD = dyn;                    // kp x XS, then D'
     double* sE = sD + kp * XS;
@@ -2345,7 +2346,7 @@ struct Engine {
     double* sX0 = wk + RC * VS;
     // rows [rb, rb + nr) of columns base .. into a buffer
     auto stage_x = [&](double* sX, int base, int rb, int nr) {
-      for (int c = warp; c < 32; c += NW) {
+      for (int c = warp; c < CW; c += NW) {
         const bool in = base + c < n;
         const int id = in ? list[base + c] : -1;
         const double* col = (id >= 0 ? Wcol(id) : I.bt) + nP + rb;
@@ -2356,9 +2357,9 @@ struct Engine {
     __syncthreads();
     if (whole) stage_vrows(sV, VS, s_vt, 0, L);
     if (whole) stage_x(sX0, 0, 0, L);
-    for (int base = 0, b = 0; base < n; base += 32, b ^= two ? 1 : 0) {
+    for (int base = 0, b = 0; base < n; base += CW, b ^= two ? 1 : 0) {
       double* sX = sX0 + b * RC * XS;
-      const int nc = min(32, n - base);
+      const int nc = min(CW, n - base);
       double acc[4][2];
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[k][0] = acc[k][1] = 0.0;
@@ -2373,21 +2374,21 @@ struct Engine {
         }
         cp_wait_all();
         __syncthreads();
-        if (two && base + 32 < n) stage_x(sX0 + (b ^ 1) * RC * XS, base + 32, 0, L);
+        if (two && base + CW < n) stage_x(sX0 + (b ^ 1) * RC * XS, base + CW, 0, L);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int t = warp + k * NW;
           if (t >= kp) break;
           // V(r, t) = 0 above row t
           double a0 = acc[k][0], a1 = acc[k][1];
-          int rr = max(0, t - rb);
-          for (; rr + 3 < nr; rr += 4) {
-            a0 = fma(sV[rr * VS + t], sX[rr * XS + lane], a0);
-            a1 = fma(sV[(rr + 1) * VS + t], sX[(rr + 1) * XS + lane], a1);
-            a0 = fma(sV[(rr + 2) * VS + t], sX[(rr + 2) * XS + lane], a0);
-            a1 = fma(sV[(rr + 3) * VS + t], sX[(rr + 3) * XS + lane], a1);
+          int rr = max(0, t - rb) + g;
+          for (; rr + 3 * G < nr; rr += 4 * G) {
+            a0 = fma(sV[rr * VS + t], sX[rr * XS + cl], a0);
+            a1 = fma(sV[(rr + G) * VS + t], sX[(rr + G) * XS + cl], a1);
+            a0 = fma(sV[(rr + 2 * G) * VS + t], sX[(rr + 2 * G) * XS + cl], a0);
+            a1 = fma(sV[(rr + 3 * G) * VS + t], sX[(rr + 3 * G) * XS + cl], a1);
           }
-          for (; rr < nr; ++rr) a0 = fma(sV[rr * VS + t], sX[rr * XS + lane], a0);
+          for (; rr < nr; rr += G) a0 = fma(sV[rr * VS + t], sX[rr * XS + cl], a0);
           acc[k][0] = a0;
           acc[k][1] = a1;
         }
@@ -2395,19 +2396,21 @@ struct Engine {
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int t = warp + k * NW;
-        if (t < kp) sD[t * XS + lane] = acc[k][0] + acc[k][1];
+        double v = acc[k][0] + acc[k][1];
+        for (int o = CW; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (t < kp) sD[t * XS + cl] = v;
       }
       __syncthreads();
-      for (int t = warp; t < kp; t += NW) {
+      for (int t = warp * G + g; t < kp; t += NW * G) {
         const double* tr = s_T + t * (t + 1) / 2;
         double e0 = 0.0, e1 = 0.0;
         int q = 0;
         for (; q + 1 <= t; q += 2) {
-          e0 = fma(tr[q], sD[q * XS + lane], e0);
-          e1 = fma(tr[q + 1], sD[(q + 1) * XS + lane], e1);
+          e0 = fma(tr[q], sD[q * XS + cl], e0);
+          e1 = fma(tr[q + 1], sD[(q + 1) * XS + cl], e1);
         }
-        if (q <= t) e0 = fma(tr[q], sD[q * XS + lane], e0);
-        sE[t * XS + lane] = e0 + e1;
+        if (q <= t) e0 = fma(tr[q], sD[q * XS + cl], e0);
+        sE[t * XS + cl] = e0 + e1;
       }
       double nrm = 0.0;
       for (int rb = 0; rb < L; rb += RC) {
@@ -2419,20 +2422,20 @@ struct Engine {
           cp_wait_all();
         }
         __syncthreads();
-        for (int rr = warp; rr < nr; rr += NW) {
+        for (int rr = warp * G + g; rr < nr; rr += NW * G) {
           const int te = min(rb + rr + 1, kp);
-          double x0 = sX[rr * XS + lane], x1 = 0.0;
+          double x0 = sX[rr * XS + cl], x1 = 0.0;
           const double* v = sV + rr * VS;
           int t = 0;
           for (; t + 3 < te; t += 4) {
-            x0 = fma(-v[t], sE[t * XS + lane], x0);
-            x1 = fma(-v[t + 1], sE[(t + 1) * XS + lane], x1);
-            x0 = fma(-v[t + 2], sE[(t + 2) * XS + lane], x0);
-            x1 = fma(-v[t + 3], sE[(t + 3) * XS + lane], x1);
+            x0 = fma(-v[t], sE[t * XS + cl], x0);
+            x1 = fma(-v[t + 1], sE[(t + 1) * XS + cl], x1);
+            x0 = fma(-v[t + 2], sE[(t + 2) * XS + cl], x0);
+            x1 = fma(-v[t + 3], sE[(t + 3) * XS + cl], x1);
           }
-          for (; t < te; ++t) x0 = fma(-v[t], sE[t * XS + lane], x0);
+          for (; t < te; ++t) x0 = fma(-v[t], sE[t * XS + cl], x0);
           x0 += x1;
-          sX[rr * XS + lane] = x0;
+          sX[rr * XS + cl] = x0;
           if (rb + rr >= kp) nrm = fma(x0, x0, nrm);
         }
         __syncthreads();
@@ -2442,7 +2445,8 @@ struct Engine {
           for (int r = lane; r < nr; r += 32) col[r] = sX[r * XS + c];
         }
       }
-      sN[warp * XS + lane] = nrm;
+      for (int o = CW; o < 32; o <<= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+      sN[warp * XS + cl] = nrm;
       __syncthreads();
       if (warp == 0 && lane < nc) {
         double v = 0.0;
@@ -3600,7 +3604,7 @@ struct Engine {
     if (narrow) {
       commit_narrow(s_T, s_vt, s_list, nl, L);
     } else if (!tc && !(tall && L > cols_rows())) {
-      commit_cols(s_T, s_vt, s_list, nl, L);
+      commit_cols(s_T, s_vt, s_list, nl, L, 5);
     } else {
       for (int base = 0; base < nl; base += CB) {
         const int nb = min(CB, nl - base);
@@ -3638,7 +3642,7 @@ struct Engine {
             continue;
           }
         }
-        commit_cols(s_T, s_vt, s_list + base, nb, L);
+        commit_cols(s_T, s_vt, s_list + base, nb, L, nb <= 8 ? 3 : 4);
       }
     }
     nP += kp;

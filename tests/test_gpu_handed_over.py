@@ -1,0 +1,57 @@
+"""Commit batches that the accuracy guard hands to FP64: they work on as many
+lanes as the batch has columns for (8 or 16), beside rows that do not fit
+shared memory whole.  Forced for every batch here.  Bar: identical passive set
+and counters, ||x - x_oracle|| <= 1e-10 ||x_oracle|| (the parity bar of every
+GPU test), and a commit phase at a quarter of the 1.26 TFLOP/s the GPU has in
+FP64 (32 lanes for the 7 and 14 columns of a CTA kept a ninth and less than a
+quarter)."""
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2108_05345_gb300 import workloads as WL
+from gpu_util import assert_parity, solve
+
+pytestmark = pytest.mark.gpu
+
+# m, n, nonzeros, k_max: 1 to 16 columns per CTA
+CASES = [(700, 130, 20, 16), (900, 700, 40, 32), (1300, 1200, 60, 48), (800, 1500, 50, 64), (1100, 2400, 60, 32)]
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_05345_gb300 import build, lhdm
+    build.build()
+    return lhdm
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_parity(L, case):
+    m, n, s, k = case
+    A, b, _ = WL.gaussian_recovery(m, n, s, 9, unit_columns=True)
+    ref = O.nnls(A, b, k_max=k, trace=True)
+    ctx = L.Context(m, n)
+    ctx.force_commit_guard(1)
+    x, P, _, info = solve(L, ctx, A, b, k_max=k)
+    assert_parity(x, P, info, ref, trace=ctx.trace())
+    ctx.close()
+
+
+@pytest.mark.parametrize("m,n", [(2048, 1024), (4096, 2048)])
+def test_rate(L, m, n):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    A = torch.rand((n, m), generator=g, device="cuda", dtype=torch.float64).t()
+    x = torch.rand(n, generator=g, device="cuda", dtype=torch.float64) * (torch.arange(n, device="cuda") % 2)
+    b = A @ x + 1e-2 * torch.randn(m, generator=g, device="cuda", dtype=torch.float64)
+    ctx = L.Context(m, n)
+    ctx.force_commit_guard(1)
+    best = 0.0
+    for _ in range(2):
+        ctx.solve(A, b, L.default_params(k_max=32))
+        ms, flops = ctx.profile()
+        best = max(best, flops["commit"] / ms["commit"] * 1e-9)
+    ctx.close()
+    assert best > 0.315, "commit at %.3f TFLOP/s" % best
