@@ -2797,6 +2797,8 @@ struct Engine {
   // Ring of pass 1: row groups per chunk, slots.
   __device__ static constexpr int p1_groups(int MT) { return MT == 1 ? 8 : 4; }
   __device__ static constexpr int p1_slots(int MT) { return MT == 2 ? 5 : MT == 4 ? 3 : 4; }
+  // chunks of one exact accumulation: 1024 rows (127^2 x 1024 < 2^24)
+  __device__ static constexpr int p1_segment(int MT) { return 128 / p1_groups(MT); }
   // The MMAs of a pass-1 chunk (16 rows per step, nks <= 4 steps) and of a
   // pass-2 tile; one thread.  Unrolled with constant descriptor steps: the
   // issuing thread's instructions must fit beside an MMA's 40 to 72 cycles.
@@ -2963,7 +2965,7 @@ struct Engine {
       }
       tc_fence_before();
     };
-    const int SEG = 128 / G1;  // chunks per exact accumulation (1024 rows)
+    const int SEG = p1_segment(MT);
     __syncthreads();            // s_Ec, sF
     // slot and use (chunk j: slot j mod NR, use j / NR) of this warp's next
     // chunk, kept by counting (a division is as long as a chunk's MMAs)
