@@ -4283,8 +4283,9 @@ struct Engine {
     // R columns round-robin over the ranks (the last positions, which take
     // the most rotations, land on different CTAs)
     const int nr_own = (zr < nrot) ? (nrot - zr + nzr - 1) / nzr : 0;
-    // rows of R^{-1}, one position after another like R's columns
-    const int ni_own = (inv_n == np && zr < np - 1) ? (np - 1 - zr + nzr - 1) / nzr : 0;
+    // rows of R^{-1}, one position after another like R's columns (kept for
+    // all positions only where the rotations came from it: never with `follow`)
+    const int ni_own = (!follow && inv_n == np && zr < np - 1) ? (np - 1 - zr + nzr - 1) / nzr : 0;
     const int nunit = nz + nr_own + ni_own;
     // the products for the chunk at stage offset t0 (one warp)
     auto chunk_products = [&](int t0, int ns) {
@@ -4542,16 +4543,15 @@ struct Engine {
         bool rlast;
         int ts;
         unit(k, 0, nrot, colp, nsu, rlast, ts);
-        if (nsu <= 0) continue;
         // an R column waits for its own chain block's rotations: that block
         // read the column from global memory before generating them
-        if (k >= nz && k < nz + nr_own && !wait_avail((nsu - 1) / DB + 1)) {
+        if (k >= nz && !wait_avail((nsu - 1) / DB + 1)) {
           ok = false;
           break;
         }
-        double carry = ldcg(colp + q + ts);
-        double nbot = (ts + lane < nsu) ? ldcg(colp + q + ts + 1 + lane) : 0.0;
-        for (int t0 = ts; t0 < nsu; t0 += 32) {
+        double carry = ldcg(colp + q);
+        double nbot = (lane < nsu) ? ldcg(colp + q + 1 + lane) : 0.0;
+        for (int t0 = 0; t0 < nsu; t0 += 32) {
           if (!wait_avail(t0 / 32 + 1)) {
             ok = false;
             break;
