@@ -125,9 +125,10 @@ const char* lhdm_status_string(int status);
  * Creates a solve context on the current CUDA device for single problems up
  * to max_m x max_n (lhdm_solve) and for batches of up to max_batch problems,
  * each at most max_m x max_n (lhdm_solve_batched; max_batch = 0: no batched
- * solves).  Allocates the single-solve workspace here (FP64, about
- * 8 * (max_m * max_n + min(max_m,max_n)^2) bytes plus O(max_m + max_n));
- * later single solves allocate nothing.  The batch workspace is sized by the
+ * solves).  Allocates the single-solve workspace here (FP64, with c =
+ * min(max_m,max_n) about 8 * (max_m * max_n + c^2 + c * min(c, 3072)) bytes
+ * plus O(max_m + max_n); where that fails, without the last term, at the cost
+ * of slower solves); later single solves allocate nothing.  The batch workspace is sized by the
  * first lhdm_solve_batched call with a given set of instances (see there).
  * *ctx receives the handle (host).
  * Errors: INVALID_ARG (sizes < 1, max_batch < 0 or ctx NULL), ALLOC, CUDA.

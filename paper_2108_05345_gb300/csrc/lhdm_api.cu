@@ -22,7 +22,7 @@ using namespace lhdm;
 struct lhdm_ctx {
   int device = 0;
   int nsm = 0;
-  int max_m = 0, max_n = 0, cap = 0, ldr = 0;
+  int max_m = 0, max_n = 0, cap = 0, ldr = 0, ldi = 0;
   ScratchLayout L{};
   char* arena = nullptr;  // the one allocation that the pointers below share
   double* dscr = nullptr;
@@ -201,6 +201,7 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
   c->ctas = c->nsm;
   c->cap = std::max(std::min(max_m, max_n), 1);
   c->ldr = (c->cap + 1) & ~1;
+  c->ldi = (std::min(c->cap, INV_ROWS) + 1) & ~1;  // a slot's row of the inverse (any slot can hold one)
   if ((max_n + c->nsm - 1) / c->nsm > CAND_LOCAL_MAX) { delete c; return LHDM_ERR_INVALID_ARG; }
   c->L = make_layout(max_m, max_n, c->nsm);
   // one allocation, carved in 256-byte granules: the words that start at zero
@@ -221,7 +222,7 @@ int lhdm_create(lhdm_ctx** out, int32_t max_m, int32_t max_n, int32_t max_batch)
                o_r = take((size_t)std::max(max_m, 1) * sizeof(double)),
                o_trace = take((size_t)6 * c->trace_cap * sizeof(int)), o_iscr = take(c->L.itotal * sizeof(int)),
                o_dscr = take(c->L.dtotal * sizeof(double)), o_R = take(nR * sizeof(double)), without = total,
-               o_Rinv = take(nR * sizeof(double));
+               o_Rinv = take((size_t)c->ldi * c->cap * sizeof(double));
   bool inv = true;
   cudaError_t e = cudaMalloc(&c->arena, total);
   if (e == cudaErrorMemoryAllocation) {
@@ -312,6 +313,7 @@ int lhdm_solve(lhdm_ctx* c, int32_t m, int32_t n, const double* A, int32_t lda, 
   I.prm = to_dev(p);
   fill_ctx_inst(c, I);
   I.Rinv = c->Rinv;
+  I.ldi = c->ldi;
   I.bar_extra = c->stall_next ? 1 : 0;
   c->stall_next = false;
   c->have_state = false;

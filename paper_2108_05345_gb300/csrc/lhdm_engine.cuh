@@ -39,6 +39,12 @@ namespace lhdm {
 
 constexpr int KM = LHDM_KMAX_LIMIT;  // 64
 constexpr int NT = 512;              // threads per CTA
+// Positions up to which R's inverse is kept.  It pays at every size measured:
+// against substitution from 2048 on, a solve that ends with 3291 positions
+// (8192 x 4096, k_max 32) takes 142 instead of 209 ms, and 4096 would take
+// another 25 % off one with 4475 (8192 x 5000).  The limit is for the memory,
+// 24 KB a position of the context's largest problem.
+constexpr int INV_ROWS = 3072;
 constexpr int NW = NT / 32;          // warps per CTA
 constexpr int PW = 2112;             // partial-sum slots per CTA (>= KM(KM+1)/2 + 16)
 // Slot ranges inside one CTA's partial row.  A range is only rewritten after
@@ -75,7 +81,7 @@ struct DevParams {
 // Everything a team needs for one instance.  Persistent fields (R, rslot,
 // order, xP, r, nP_out) survive the solve for the adjoint.
 struct Inst {
-  int m, n, lda, cap, ldw, ldr;
+  int m, n, lda, cap, ldw, ldr, ldi;
   const double* A;
   const double* b;
   double* x_out;
@@ -88,7 +94,7 @@ struct Inst {
   double* xP;
   double* r;
   int* nP_out;
-  double* Rinv;   // inverse of R, row of position p in slot rslot[p] (ld ldr; null: not kept)
+  double* Rinv;   // inverse of R up to INV_ROWS positions, row of position p in slot rslot[p] (ld ldi; null: not kept)
   // scratch
   double* W;
   double* bt;

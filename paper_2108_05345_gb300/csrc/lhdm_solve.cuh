@@ -1857,10 +1857,10 @@ struct Engine {
   // step) or, with a barrier of its own, at the end of the inner loop; it
   // costs 2.4 % of a one-column solve at 2048 x 1024 (57.7 -> 59.2 ms) and of
   // a conditioned one (52.9 -> 54.2 ms), 0.9 % at 4096 x 2048.
-  static constexpr int INV_MIN = 2 * TB, INV_ROWS = 3072;
+  static constexpr int INV_MIN = 2 * TB;
   static constexpr int INV_BITS = 26;
   int chk_ep = 0;  // the corrected solve whose test is still to be read (0: none)
-  __device__ __forceinline__ double* Irow(int p) const { return I.Rinv + (size_t)ldcg(I.rslot + p) * I.ldr; }
+  __device__ __forceinline__ double* Irow(int p) const { return I.Rinv + (size_t)ldcg(I.rslot + p) * I.ldi; }
 
   // yP (+)= R^{-1} v on positions [0, np), a warp per row.
   __device__ void inv_product(int np, const double* v, bool add) {
@@ -2148,7 +2148,7 @@ struct Engine {
   __device__ void inv_rotations(int q, int np, int nrot, int ep) {
     double* sv = dyn;  // v(q .. np - 1)
     __shared__ double sh[32];
-    const double* v = I.Rinv + (size_t)ldcg(I.rslot + np - 1) * I.ldr + q;
+    const double* v = I.Rinv + (size_t)ldcg(I.rslot + np - 1) * I.ldi + q;
     __syncthreads();
     for (int j = tid; j <= nrot; j += NT) sv[j] = ldcg(v + j);
     __syncthreads();
