@@ -2752,7 +2752,7 @@ struct Engine {
   // Pass 2 has no guard: an element whose products all lie far below its row's
   // and its column's scale keeps fewer bits than in FP64 (its error is at most
   // (3 kp + 2) 2^(Er + Ee - 57)).  Measured error of x against refined
-  // solutions, geometric means over 66 solutions, with 33 to 64 reflectors in
+  // solutions, geometric means over 53 solutions, with 33 to 64 reflectors in
   // digits and in FP64: dense 1.8e-14 and 2.3e-14, signed 1.5e-15 and
   // 1.7e-15, conditioned (1e5, 1e6) 5.9e-13, l1 1.5e-15 and recovery 2.0e-15
   // on both; every block in FP64: 2.3e-14, 1.7e-15, 6.0e-13, 1.5e-15, 2.1e-15.

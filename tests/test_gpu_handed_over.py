@@ -2,9 +2,9 @@
 lanes as the batch has columns for (8 or 16), beside rows that do not fit
 shared memory whole.  Forced for every batch here.  Bar: identical passive set
 and counters, ||x - x_oracle|| <= 1e-10 ||x_oracle|| (the parity bar of every
-GPU test), and a commit phase at a quarter of the 1.26 TFLOP/s the GPU has in
-FP64 (32 lanes for the 7 and 14 columns of a CTA kept a ninth and less than a
-quarter)."""
+GPU test), and the commit phase's rate: 0.37 and 0.59 TFLOP/s were measured
+with 7 and 14 columns per CTA, 0.14 and 0.28 with 32 lanes for them; the bars
+lie between."""
 import pytest
 import torch
 
@@ -39,8 +39,8 @@ def test_parity(L, case):
     ctx.close()
 
 
-@pytest.mark.parametrize("m,n", [(2048, 1024), (4096, 2048)])
-def test_rate(L, m, n):
+@pytest.mark.parametrize("m,n,bar", [(2048, 1024, 0.22), (4096, 2048, 0.4)])
+def test_rate(L, m, n, bar):
     g = torch.Generator(device="cuda")
     g.manual_seed(3)
     A = torch.rand((n, m), generator=g, device="cuda", dtype=torch.float64).t()
@@ -54,4 +54,4 @@ def test_rate(L, m, n):
         ms, flops = ctx.profile()
         best = max(best, flops["commit"] / ms["commit"] * 1e-9)
     ctx.close()
-    assert best > 0.315, "commit at %.3f TFLOP/s" % best
+    assert best > bar, "commit at %.3f TFLOP/s" % best
