@@ -19,7 +19,8 @@ pytestmark = pytest.mark.gpu
 # m, n, nonzeros, k_max
 CASES = [(17000, 120, 12, 8), (17000, 400, 20, 16), (16900, 1000, 30, 32), (17000, 1400, 40, 40), (17500, 2300, 30, 32),
          (9000, 900, 20, 4)]
-ONE_CTA = [(17000, 40, 10, 8), (16500, 33, 12, 12), (9000, 50, 10, 4)]
+# the same kernel takes the small ones of a mixed batch
+ONE_CTA = [(17000, 40, 10, 8), (600, 300, 40, 8), (16500, 33, 12, 12), (9000, 50, 10, 4), (700, 400, 30, 4), (90, 60, 9, 4)]
 
 
 @pytest.fixture(scope="module")
